@@ -184,7 +184,7 @@ typedef struct {
 enum {
     PT_MODE_AUTO = 0,           /* pick per the autotuned table (pt_autotune) */
     PT_MODE_WAVEFRONT = 1,      /* queue-driven kernels per bounce (raygen/trace/sort/shade/shadow) */
-    PT_MODE_MEGAKERNEL = 2      /* persistent kernel, one path per thread, work-queue fetch */
+    PT_MODE_MEGAKERNEL = 2      /* one kernel, one thread per path, each path to its end */
 };
 
 typedef struct {

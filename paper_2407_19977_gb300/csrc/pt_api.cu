@@ -158,7 +158,7 @@ static void free_scene(pt_scene* s) {
     if (!s) return;
     void* ptrs[] = {s->d_vertices, s->d_indices, s->d_matids, s->d_tris_raw, s->d_tris, s->d_nodes,
                     s->d_mats, s->d_fuzz, s->d_quads, s->d_quads_raw, s->d_env, s->d_env_marg, s->d_env_cond,
-                    s->d_env_wtex, s->d_env_total, s->d_env_guide, s->d_err, s->d_stats, s->d_head};
+                    s->d_env_wtex, s->d_env_total, s->d_env_guide, s->d_err, s->d_stats};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     pt_free_wave(s->wave);
@@ -240,7 +240,6 @@ extern "C" pt_status pt_scene_create(const float* vertices, uint32_t n_vertices,
     TRY(cudaMalloc(&s->d_quads_raw, std::max<uint32_t>(n_lights, 1) * 13 * sizeof(float)));
     TRY(cudaMalloc(&s->d_err, 16 * sizeof(uint32_t)));
     TRY(cudaMalloc(&s->d_stats, ST_COUNT * sizeof(unsigned long long)));
-    TRY(cudaMalloc(&s->d_head, 64 * sizeof(uint32_t)));
     TRY(cudaMemsetAsync(s->d_err, 0, 16 * sizeof(uint32_t), st));
     TRY(cudaMemsetAsync(s->d_stats, 0, ST_COUNT * sizeof(unsigned long long), st));
     if (n_triangles > 0) {

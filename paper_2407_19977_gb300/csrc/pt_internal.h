@@ -117,7 +117,6 @@ struct pt_scene {
     float lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     uint32_t* d_err = nullptr;
     unsigned long long* d_stats = nullptr;
-    uint32_t* d_head = nullptr;      // persistent work-queue heads (scratch)
     bool built = false;
     WaveBuffers wave;
     cudaStream_t last_stream = nullptr;

@@ -45,56 +45,69 @@ struct PixelCounters {
     unsigned long long ext, shadow, nan, rr, paths;
 };
 
-__device__ __forceinline__ void render_pixel(const DJob& J, uint32_t lp, PixelCounters& cnt) {
-    const uint32_t px = J.x0 + lp % J.cw, py = J.y0 + lp / J.cw;
+// radiance of sample s of pixel (px, py), with non-finite results dropped and counted
+template <bool FUZZ>
+__device__ __forceinline__ float3 render_sample(const DJob& J, uint32_t px, uint32_t py, uint32_t s, PixelCounters& cnt) {
     const uint32_t p = py * J.cam.width + px;
     const uint32_t k0 = (uint32_t)J.seed, k1 = (uint32_t)(J.seed >> 32);
+    float3 o, d;
+    camera_ray_ps(J.cam, px, py, p, s, k0, k1, o, d);
+    PathState ps;
+    ps.beta = splat3(1.0f);
+    ps.L = splat3(0.0f);
+    ps.prev_pdf = -1.0f;
+    for (uint32_t k = 0;; ++k) {
+        HitRec h;
+        trace_closest(J.S, o, d, __int_as_float(0x7f800000), h);
+        cnt.ext++;
+        VertexRng rng;
+        rng.p = p; rng.s = s; rng.k = k; rng.k0 = k0; rng.k1 = k1;
+        ShadeOut so;
+        const int r = shade_vertex<false, FUZZ>(J.S, h, o, d, k, J.max_depth, J.flags, rng, ps, so);
+        if (so.has_shadow) {
+            cnt.shadow++;
+            if (!trace_any(J.S, so.sh.o, so.sh.d, so.sh.tmax)) ps.L = ps.L + so.sh.contrib;
+        }
+        if (r == SHADE_END) {
+            if (so.rr_end) cnt.rr++;
+            break;
+        }
+        o = so.next_o;
+        d = so.next_d;
+    }
+    cnt.paths++;
+    float3 L = ps.L;
+    if (!isfinite(L.x) || !isfinite(L.y) || !isfinite(L.z)) {
+        cnt.nan++;
+        L = splat3(0.0f);
+    }
+    return L;
+}
+
+__device__ __forceinline__ void render_pixel(const DJob& J, uint32_t lp, PixelCounters& cnt) {
     float* sp = J.sum + 3ull * lp;
     float* cp = J.comp + 3ull * lp;
     float s0 = sp[0], s1 = sp[1], s2 = sp[2], c0 = cp[0], c1 = cp[1], c2 = cp[2];
     for (uint32_t i = 0; i < J.spp; ++i) {
-        const uint32_t s = J.s0 + i;
-        float3 o, d;
-        camera_ray_ps(J.cam, px, py, p, s, k0, k1, o, d);
-        PathState ps;
-        ps.beta = splat3(1.0f);
-        ps.L = splat3(0.0f);
-        ps.prev_pdf = -1.0f;
-        for (uint32_t k = 0;; ++k) {
-            HitRec h;
-            trace_closest(J.S, o, d, __int_as_float(0x7f800000), h);
-            cnt.ext++;
-            VertexRng rng;
-            rng.p = p; rng.s = s; rng.k = k; rng.k0 = k0; rng.k1 = k1;
-            ShadeOut so;
-            const int r = shade_vertex(J.S, h, o, d, k, J.max_depth, J.flags, rng, ps, so);
-            if (so.has_shadow) {
-                cnt.shadow++;
-                if (!trace_any(J.S, so.sh.o, so.sh.d, so.sh.tmax)) ps.L = ps.L + so.sh.contrib;
-            }
-            if (r == SHADE_END) {
-                if (so.rr_end) cnt.rr++;
-                break;
-            }
-            o = so.next_o;
-            d = so.next_d;
-        }
-        cnt.paths++;
-        float3 L = ps.L;
-        if (!isfinite(L.x) || !isfinite(L.y) || !isfinite(L.z)) {
-            cnt.nan++;
-            L = splat3(0.0f);
-        }
-        if (J.sample_out) {
-            float* o3 = J.sample_out + 3ull * ((uint64_t)lp * J.spp + i);
-            o3[0] = L.x; o3[1] = L.y; o3[2] = L.z;
-        }
+        const float3 L = render_sample<true>(J, J.x0 + lp % J.cw, J.y0 + lp / J.cw, J.s0 + i, cnt);
         kahan_add(s0, c0, L.x);
         kahan_add(s1, c1, L.y);
         kahan_add(s2, c2, L.z);
     }
     sp[0] = s0; sp[1] = s1; sp[2] = s2;
     cp[0] = c0; cp[1] = c1; cp[2] = c2;
+}
+
+__device__ __forceinline__ void megakernel_stats(const DJob& J, const PixelCounters& cnt) {
+    const unsigned long long e = warp_sum_u64(cnt.ext), sh = warp_sum_u64(cnt.shadow),
+                             nn = warp_sum_u64(cnt.nan), rr = warp_sum_u64(cnt.rr), pa = warp_sum_u64(cnt.paths);
+    if (lane_id() == 0) {
+        atomicAdd(&J.stats[ST_EXT], e);
+        atomicAdd(&J.stats[ST_SHADOW], sh);
+        if (nn) atomicAdd(&J.stats[ST_NAN], nn);
+        if (rr) atomicAdd(&J.stats[ST_RR], rr);
+        atomicAdd(&J.stats[ST_PATHS], pa);
+    }
 }
 
 __device__ __forceinline__ void megakernel_item(const DJob& J, uint32_t item, uint32_t tile_pixels) {
@@ -104,15 +117,7 @@ __device__ __forceinline__ void megakernel_item(const DJob& J, uint32_t item, ui
     const uint32_t pe = min(pb + tile_pixels, npix);
     PixelCounters cnt = {0, 0, 0, 0, 0};
     for (uint32_t lp = pb + lane; lp < pe; lp += 32) render_pixel(J, lp, cnt);
-    const unsigned long long e = warp_sum_u64(cnt.ext), sh = warp_sum_u64(cnt.shadow),
-                             nn = warp_sum_u64(cnt.nan), rr = warp_sum_u64(cnt.rr), pa = warp_sum_u64(cnt.paths);
-    if (lane == 0) {
-        atomicAdd(&J.stats[ST_EXT], e);
-        atomicAdd(&J.stats[ST_SHADOW], sh);
-        if (nn) atomicAdd(&J.stats[ST_NAN], nn);
-        if (rr) atomicAdd(&J.stats[ST_RR], rr);
-        atomicAdd(&J.stats[ST_PATHS], pa);
-    }
+    megakernel_stats(J, cnt);
 }
 
 // warps pop work items until the queue is empty; an item is a tile of pixels of one job
@@ -136,13 +141,59 @@ __global__ void __launch_bounds__(128) k_megakernel(const DJob* __restrict__ job
     }
 }
 
-__global__ void __launch_bounds__(128) k_megakernel_one(const __grid_constant__ DJob job, uint32_t total_items,
-                                                        uint32_t tile_pixels, uint32_t* head) {
-    for (;;) {
-        const uint32_t item = pop_item(head);
-        if (item >= total_items) break;
-        megakernel_item(job, item, tile_pixels);
+// Bound by the latency of a path's chain of node loads; the measure is to have every path of a
+// small frame in flight at once.  A lane per pixel that loops over the samples, 64 pixels a
+// warp, left a 64 x 64 frame of 16 samples to 64 warps: 3.30 ms, now 0.18 ms (Cornell box,
+// depth 4).
+// One job, one thread per path: a block renders `pix` consecutive pixels of the window, S samples
+// of each side by side (thread = pixel * S + sample), and every pixel's radiances are then
+// added in sample order by one thread, so the sums are those of a serial loop over samples.
+constexpr uint32_t PATH_THREADS = 128;
+
+template <bool FUZZ>
+__global__ void __launch_bounds__(PATH_THREADS, 4) k_megakernel_one(const __grid_constant__ DJob job, uint32_t S,
+                                                                    uint32_t pix) {
+    __shared__ float rad[3][PATH_THREADS];
+    const uint32_t t = threadIdx.x, npix = job.cw * job.ch;
+    const uint32_t p0 = blockIdx.x * pix;
+    const uint32_t lp = p0 + t / S, q = t % S;
+    const bool mine = t / S < pix && lp < npix;
+    // the thread that adds up pixel p0 + t
+    const bool adds = t < pix && p0 + t < npix;
+    float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f, c0 = 0.0f, c1 = 0.0f, c2 = 0.0f;
+    float* sp = job.sum + 3ull * (p0 + t);
+    float* cp = job.comp + 3ull * (p0 + t);
+    if (adds) {
+        s0 = sp[0]; s1 = sp[1]; s2 = sp[2];
+        c0 = cp[0]; c1 = cp[1]; c2 = cp[2];
     }
+    PixelCounters cnt = {0, 0, 0, 0, 0};
+    for (uint32_t i0 = 0; i0 < job.spp; i0 += S) {
+        const uint32_t i = i0 + q;
+        if (mine && i < job.spp) {
+            const float3 L = render_sample<FUZZ>(job, job.x0 + lp % job.cw, job.y0 + lp / job.cw, job.s0 + i, cnt);
+            if (job.sample_out) {
+                float* o3 = job.sample_out + 3ull * ((uint64_t)lp * job.spp + i);
+                o3[0] = L.x; o3[1] = L.y; o3[2] = L.z;
+            }
+            rad[0][t] = L.x; rad[1][t] = L.y; rad[2][t] = L.z;
+        }
+        __syncthreads();
+        if (adds) {
+            const uint32_t n = min(S, job.spp - i0);
+            for (uint32_t k = 0; k < n; ++k) {
+                kahan_add(s0, c0, rad[0][t * S + k]);
+                kahan_add(s1, c1, rad[1][t * S + k]);
+                kahan_add(s2, c2, rad[2][t * S + k]);
+            }
+        }
+        __syncthreads();
+    }
+    if (adds) {
+        sp[0] = s0; sp[1] = s1; sp[2] = s2;
+        cp[0] = c0; cp[1] = c1; cp[2] = c2;
+    }
+    megakernel_stats(job, cnt);
 }
 
 static int g_mk_blocks_per_sm = 0;
@@ -160,14 +211,14 @@ static uint32_t megakernel_grid(uint32_t total_items, uint32_t blocks_per_sm) {
 }
 
 // one job: the job travels as a kernel parameter, nothing is staged in device memory
-static pt_status launch_megakernel_one(DJob job, uint32_t tile_pixels, uint32_t blocks_per_sm, cudaStream_t st,
-                                       uint32_t* d_head, uint64_t* launches) {
-    job.tile_begin = 0;
-    job.n_tiles = (job.cw * job.ch + tile_pixels - 1) / tile_pixels;
-    if (job.n_tiles == 0) return PT_OK;
-    PT_CUDA_TRY(cudaMemsetAsync(d_head, 0, sizeof(uint32_t), st));
-    PT_LAUNCH(k_megakernel_one, megakernel_grid(job.n_tiles, blocks_per_sm), 128, 0, st, job, job.n_tiles,
-              tile_pixels, d_head);
+static pt_status launch_megakernel_one(const DJob& job, uint32_t block_size, bool fuzz, cudaStream_t st,
+                                       uint64_t* launches) {
+    const uint32_t npix = job.cw * job.ch;
+    const uint32_t threads = block_size ? std::min(std::max(32u, block_size & ~31u), PATH_THREADS) : PATH_THREADS;
+    const uint32_t S = std::min(job.spp, 32u), pix = threads / S;
+    const uint32_t grid = (npix + pix - 1) / pix;
+    if (fuzz) PT_LAUNCH(k_megakernel_one<true>, grid, threads, 0, st, job, S, pix);
+    else PT_LAUNCH(k_megakernel_one<false>, grid, threads, 0, st, job, S, pix);
     (*launches)++;
     PT_CUDA_TRY(cudaGetLastError());
     return PT_OK;
@@ -1842,6 +1893,34 @@ static DJob make_job(pt_scene* s, const pt_camera& cam, uint32_t x0, uint32_t y0
 }
 
 
+// PT_MODE_AUTO without a tuned schedule: one thread per path for few paths, the wavefront for
+// many.  The path kernel is one launch but keeps a lane for a path to its end, so it loses once
+// there are paths to refill the lanes with.  Measured, path kernel against wavefront in ms, at
+// 65,536 / 131,072 / 160,000 / 320,000 / 524,288 paths: Cornell box 0.18 / 0.32 / 0.38 / 0.75 /
+// 1.23 against 0.33 / 0.34 / 0.38 / 0.50 / 0.65, 50k-triangle CAD model 0.62 / 0.82 / 0.98 /
+// 1.55 / 2.38 against 0.78 / 0.96 / 1.08 / 1.24 / 1.52, glass scene 0.50 / 0.69 / 0.77 / 1.31 /
+// 2.05 against 0.76 / 0.92 / 0.97 / 1.20 / 1.44.
+constexpr uint64_t AUTO_WAVE_PATHS = 1u << 18;
+
+static uint32_t auto_mode(const pt_render_opts& o, uint32_t npix, uint32_t spp, cudaStream_t st) {
+    if (o.nrc) return PT_MODE_WAVEFRONT;
+    const bool few = (uint64_t)npix * spp < AUTO_WAVE_PATHS;
+    if (npix >= (1u << 16)) {
+        // options that only the wavefront has keep it
+        const bool wave_opts = o.use_graph || o.kernel_ms || o.wave_paths || o.tail_paths || o.tail_bounce ||
+                               o.traversal || o.sort_by_material >= 0 || (o.flags & FLAG_COUNT);
+        return few && !wave_opts ? PT_MODE_MEGAKERNEL : PT_MODE_WAVEFRONT;
+    }
+    if (few) return PT_MODE_MEGAKERNEL;
+    // a small frame that is being captured allocates nothing: the path kernel needs no buffers
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return PT_MODE_MEGAKERNEL;
+    }
+    return cap == cudaStreamCaptureStatusNone ? PT_MODE_WAVEFRONT : PT_MODE_MEGAKERNEL;
+}
+
 extern "C" pt_status pt_render(pt_scene* s, const pt_camera* camera, uint32_t spp, uint32_t max_depth, uint64_t seed,
                                pt_accum* acc, const pt_render_opts* opts, void* cuda_stream) {
     PT_CHECK_ARG(s && camera && acc, "NULL argument");
@@ -1889,17 +1968,22 @@ extern "C" pt_status pt_render(pt_scene* s, const pt_camera* camera, uint32_t sp
             o.traversal = s->tuned_opts.traversal;
             o.tail_bounce = s->tuned_opts.tail_bounce;
         } else {
-            mode = (o.nrc || (uint64_t)acc->width * acc->height >= (1u << 16)) ? PT_MODE_WAVEFRONT : PT_MODE_MEGAKERNEL;
+            mode = auto_mode(o, acc->width * acc->height, spp, st);
         }
         if (o.restir) mode = PT_MODE_WAVEFRONT;
     }
     pt_status r;
     if (mode == PT_MODE_WAVEFRONT) {
         r = render_wavefront(s, *camera, spp, max_depth, seed, acc, o, st);
-    } else {
-        const uint32_t tile = o.block_size ? std::max(32u, o.block_size & ~31u) : 64u;
+        // a small frame that AUTO sent here renders without the wave's buffers if there is no room
+        if (r == PT_ERR_OOM && o.mode == PT_MODE_AUTO && !o.nrc && !o.restir && acc->width * acc->height < (1u << 16)) {
+            cudaGetLastError();
+            mode = PT_MODE_MEGAKERNEL;
+        }
+    }
+    if (mode != PT_MODE_WAVEFRONT) {
         r = launch_megakernel_one(make_job(s, *camera, o.crop_x0, o.crop_y0, acc, spp, max_depth, seed, o.flags,
-                                           o.sample_out), tile, 0, st, s->d_head, &s->launches);
+                                           o.sample_out), o.block_size, s->has_fuzz, st, &s->launches);
     }
     if (r == PT_OK) acc->spp_done += spp;
     return r;
