@@ -12,38 +12,21 @@
 
 #define LEAF_BIT 0x80000000u
 
-__device__ __forceinline__ uint32_t f2ord_b(float f) {
-    const uint32_t b = __float_as_uint(f);
-    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
-}
-__device__ __forceinline__ float ord2f_b(uint32_t u) {
-    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
-}
-
 __device__ __forceinline__ float3 tri_centroid(const float4* t, uint32_t i) {
     const float4 a = t[3u * i], b = t[3u * i + 1], c = t[3u * i + 2];
     return mk3((a.x + b.x + c.x) * (1.0f / 3.0f), (a.y + b.y + c.y) * (1.0f / 3.0f), (a.z + b.z + c.z) * (1.0f / 3.0f));
 }
 
-__global__ void k_centroid_bounds(const float4* tris, uint32_t n, uint32_t* cb) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    float lo[3] = {3e38f, 3e38f, 3e38f}, hi[3] = {-3e38f, -3e38f, -3e38f};
-    if (i < n) {
+// One atomic per block and bound: six atomics per warp on six addresses were serialised in L2
+// (1.07M triangles: 134 us, now 9).
+__global__ void __launch_bounds__(256) k_centroid_bounds(const float4* tris, uint32_t n, uint32_t* cb) {
+    float3 lo = mk3(3e38f, 3e38f, 3e38f), hi = mk3(-3e38f, -3e38f, -3e38f);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const float3 c = tri_centroid(tris, i);
-        lo[0] = hi[0] = c.x; lo[1] = hi[1] = c.y; lo[2] = hi[2] = c.z;
+        lo = mk3(fminf(lo.x, c.x), fminf(lo.y, c.y), fminf(lo.z, c.z));
+        hi = mk3(fmaxf(hi.x, c.x), fmaxf(hi.y, c.y), fmaxf(hi.z, c.z));
     }
-    for (int a = 0; a < 3; ++a) {
-        for (int off = 16; off > 0; off >>= 1) {
-            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], off));
-            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], off));
-        }
-    }
-    if ((threadIdx.x & 31) == 0) {
-        for (int a = 0; a < 3; ++a) {
-            atomicMin(&cb[a], f2ord_b(lo[a]));
-            atomicMax(&cb[3 + a], f2ord_b(hi[a]));
-        }
-    }
+    block_bounds(lo, hi, cb);
 }
 
 __device__ __forceinline__ uint64_t spread3(uint32_t v) {
@@ -62,7 +45,7 @@ __global__ void k_morton(const float4* tris, uint32_t n, const uint32_t* cb, uin
     const float3 c = tri_centroid(tris, i);
     float q[3];
     for (int a = 0; a < 3; ++a) {
-        const float lo = ord2f_b(cb[a]), hi = ord2f_b(cb[3 + a]);
+        const float lo = ord2f(cb[a]), hi = ord2f(cb[3 + a]);
         const float ext = hi - lo;
         const float t = ext > 0.0f ? (comp3(c, a) - lo) / ext : 0.5f;
         q[a] = fminf(fmaxf(t * 2097152.0f, 0.0f), 2097151.0f);
@@ -89,36 +72,55 @@ __global__ void k_rs_hist(const uint64_t* keys, uint32_t n, int shift, uint32_t*
     hist[threadIdx.x * nblocks + blockIdx.x] = h[threadIdx.x];
 }
 
-// exclusive scan of m counters by one block of 1024 threads
-__global__ void k_rs_scan(uint32_t* data, uint32_t m) {
-    __shared__ uint32_t part[1024];
-    const uint32_t per = (m + 1023) / 1024;
-    const uint32_t b = threadIdx.x * per, e = min(b + per, m);
-    uint32_t sum = 0;
-    for (uint32_t i = b; i < e; ++i) sum += data[i];
-    part[threadIdx.x] = sum;
-    __syncthreads();
-    for (int off = 1; off < 1024; off <<= 1) {
-        const uint32_t v = threadIdx.x >= (uint32_t)off ? part[threadIdx.x - off] : 0u;
+// exclusive scan of each digit's block counts, one block per digit; the digit's total goes to
+// total[digit] and the scatter adds the digits' bases.  (One block over all 256 * nblocks
+// counters took 55 us a pass at 1.07M triangles, as long as the scatter itself; this takes 4.)
+__global__ void __launch_bounds__(256) k_rs_scan(uint32_t* hist, uint32_t nblocks, uint32_t* total) {
+    __shared__ uint32_t wsum[8];
+    uint32_t* row = hist + (size_t)blockIdx.x * nblocks;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t run = 0;
+    for (uint32_t b0 = 0; b0 < nblocks; b0 += 256) {
+        const uint32_t i = b0 + threadIdx.x;
+        const uint32_t v = i < nblocks ? row[i] : 0u;
+        uint32_t x = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        if (lane == 31) wsum[warp] = x;
         __syncthreads();
-        part[threadIdx.x] += v;
+        uint32_t before = run, all = 0;
+        for (int w = 0; w < 8; ++w) {
+            if (w < warp) before += wsum[w];
+            all += wsum[w];
+        }
+        if (i < nblocks) row[i] = before + x - v;
+        run += all;
         __syncthreads();
     }
-    uint32_t run = part[threadIdx.x] - sum;
-    for (uint32_t i = b; i < e; ++i) {
-        const uint32_t v = data[i];
-        data[i] = run;
-        run += v;
-    }
+    if (threadIdx.x == 0) total[blockIdx.x] = run;
 }
 
 // stable scatter: tile order = round-major, then thread; ranks from warp match + per-warp counts
 __global__ void k_rs_scatter(const uint64_t* kin, const uint32_t* vin, uint64_t* kout, uint32_t* vout, uint32_t n,
-                             int shift, const uint32_t* hist, uint32_t nblocks) {
+                             int shift, const uint32_t* hist, const uint32_t* total, uint32_t nblocks) {
     __shared__ uint32_t base[256];
     __shared__ uint32_t wcnt[RS_THREADS / 32][256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    base[tid] = hist[tid * nblocks + blockIdx.x];
+    // the digits' bases: exclusive scan of their totals
+    base[tid] = total[tid];
+    __syncthreads();
+    for (int off = 1; off < 256; off <<= 1) {
+        const uint32_t v = tid >= off ? base[tid - off] : 0u;
+        __syncthreads();
+        base[tid] += v;
+        __syncthreads();
+    }
+    const uint32_t digit_base = base[tid] - total[tid];
+    __syncthreads();
+    base[tid] = digit_base + hist[tid * nblocks + blockIdx.x];
     const uint32_t lt = (1u << lane) - 1u;
     for (int r = 0; r < RS_ROUNDS; ++r) {
         const uint32_t idx = blockIdx.x * RS_TILE + r * RS_THREADS + tid;
@@ -331,6 +333,15 @@ constexpr int PLOC_THREADS = 256;
 constexpr int PLOC_SCAN_ITEMS = 4;                      // per thread of the block scan
 constexpr int PLOC_SCAN_TILE = PLOC_THREADS * PLOC_SCAN_ITEMS;
 
+// The rounds run without the host: round r reads its cluster count and the merges before it
+// from state r and k_ploc_scan_top writes state r + 1 (a ring, read back every PLOC_BATCH
+// rounds).  Once at most PLOC_TAIL clusters are left the remaining rounds are many and tiny
+// (108 of 145 for a 1.07M-triangle CAD model) and one block runs them all in shared memory.
+constexpr uint32_t PLOC_BATCH = 4, PLOC_TAIL = 2048, PLOC_TAIL_THREADS = 1024;
+struct PlocState {
+    uint32_t m, merged;      // clusters, merges so far
+};
+
 struct Clusters {
     uint32_t* ref;      // LEAF_BIT | triangle id, or binary node index
     uint32_t* cnt;      // triangles below
@@ -354,8 +365,10 @@ __global__ void k_ploc_init(const float4* tris, const uint32_t* perm, uint32_t n
 }
 
 // nearest neighbour of each of the m clusters within the window (lowest index on equal area)
-__global__ void __launch_bounds__(PLOC_THREADS) k_ploc_nn(Clusters c, uint32_t m, uint32_t* nn) {
+__global__ void __launch_bounds__(PLOC_THREADS) k_ploc_nn(Clusters c, const PlocState* st, uint32_t* nn) {
     __shared__ float4 slo[PLOC_THREADS + 2 * PLOC_R], shi[PLOC_THREADS + 2 * PLOC_R];
+    const uint32_t m = st->m;
+    if (m <= PLOC_TAIL || blockIdx.x * PLOC_THREADS >= m) return;
     const int base = (int)(blockIdx.x * PLOC_THREADS) - PLOC_R;
     for (int k = threadIdx.x; k < PLOC_THREADS + 2 * PLOC_R; k += PLOC_THREADS) {
         const int g = base + k;
@@ -390,8 +403,10 @@ __device__ __forceinline__ uint64_t ploc_flag(const uint32_t* nn, uint32_t m, ui
     return i < j ? ((1ull << 32) | 1ull) : 0ull;
 }
 
-__global__ void __launch_bounds__(PLOC_THREADS) k_ploc_scan(const uint32_t* nn, uint32_t m, uint64_t* pre,
+__global__ void __launch_bounds__(PLOC_THREADS) k_ploc_scan(const uint32_t* nn, const PlocState* st, uint64_t* pre,
                                                             uint64_t* block_sum) {
+    const uint32_t m = st->m;
+    if (m <= PLOC_TAIL || blockIdx.x * PLOC_SCAN_TILE >= m) return;
     __shared__ uint64_t warp_sum[PLOC_THREADS / 32];
     const uint32_t t0 = blockIdx.x * PLOC_SCAN_TILE + threadIdx.x * PLOC_SCAN_ITEMS;
     uint64_t v[PLOC_SCAN_ITEMS], run = 0;
@@ -421,8 +436,14 @@ __global__ void __launch_bounds__(PLOC_THREADS) k_ploc_scan(const uint32_t* nn, 
     if (threadIdx.x == PLOC_THREADS - 1) block_sum[blockIdx.x] = before + x;
 }
 
-// exclusive scan of nb block totals by one block; the grand total goes to data[nb]
-__global__ void k_ploc_scan_top(uint64_t* data, uint32_t nb) {
+// exclusive scan of the block totals by one block; the grand total makes the next state
+__global__ void k_ploc_scan_top(uint64_t* data, const PlocState* st, PlocState* next) {
+    const uint32_t m = st->m;
+    if (m <= PLOC_TAIL) {
+        if (threadIdx.x == 0) *next = *st;
+        return;
+    }
+    const uint32_t nb = (m + PLOC_SCAN_TILE - 1) / PLOC_SCAN_TILE;
     __shared__ uint64_t part[1024];
     const uint32_t per = (nb + 1023) / 1024;
     const uint32_t b = threadIdx.x * per, e = min(b + per, nb);
@@ -442,16 +463,20 @@ __global__ void k_ploc_scan_top(uint64_t* data, uint32_t nb) {
         data[i] = run;
         run += v;
     }
-    if (threadIdx.x == 1023) data[nb] = part[1023];
+    if (threadIdx.x == 1023) {
+        next->m = (uint32_t)(part[1023] & 0xffffffffull);
+        next->merged = st->merged + (uint32_t)(part[1023] >> 32);
+    }
 }
 
 // survivors to their compacted position; a mutual pair becomes binary node
 // n - 2 - (merged_before + its rank among this round's merges)
-__global__ void k_ploc_compact(Clusters a, Clusters b, const uint32_t* nn, uint32_t m, const uint64_t* pre,
-                               const uint64_t* block_pre, uint32_t n, uint32_t merged_before, uint32_t* left,
+__global__ void k_ploc_compact(Clusters a, Clusters b, const uint32_t* nn, const PlocState* st, const uint64_t* pre,
+                               const uint64_t* block_pre, uint32_t n, uint32_t* left,
                                uint32_t* right, uint32_t* count, float4* blo, float4* bhi, DpArrays D) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= m) return;
+    const uint32_t m = st->m, merged_before = st->merged;
+    if (m <= PLOC_TAIL || i >= m) return;
     const uint64_t f = ploc_flag(nn, m, i);
     if (f == 0ull) return;
     const uint64_t p = pre[i] + block_pre[i / PLOC_SCAN_TILE];
@@ -486,26 +511,165 @@ __global__ void k_ploc_compact(Clusters a, Clusters b, const uint32_t* nn, uint3
 // top-down layout of the nodes [lo, hi] (one round's merges; their parents are done): each
 // node's range starts at first[node], its left subtree first; leaves take their position in
 // perm and their child reference becomes LEAF_BIT | position
-__global__ void k_ploc_layout(uint32_t lo, uint32_t hi, uint32_t* left, uint32_t* right, const uint32_t* count,
-                              uint32_t* first, uint32_t* last, uint32_t* perm) {
-    const uint32_t k = lo + blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > hi) return;
-    const uint32_t f = first[k];
-    const uint32_t L = left[k], R = right[k];
-    const uint32_t cl = (L & LEAF_BIT) ? 1u : count[L];
+struct PlocTree {
+    uint32_t *left, *right, *count, *first, *last, *perm;
+    float4 *blo, *bhi;
+};
+
+__device__ __forceinline__ void ploc_layout_node(const PlocTree& T, uint32_t k) {
+    const uint32_t f = T.first[k];
+    const uint32_t L = T.left[k], R = T.right[k];
+    const uint32_t cl = (L & LEAF_BIT) ? 1u : T.count[L];
     if (L & LEAF_BIT) {
-        perm[f] = L & ~LEAF_BIT;
-        left[k] = LEAF_BIT | f;
+        T.perm[f] = L & ~LEAF_BIT;
+        T.left[k] = LEAF_BIT | f;
     } else {
-        first[L] = f;
+        T.first[L] = f;
     }
     if (R & LEAF_BIT) {
-        perm[f + cl] = R & ~LEAF_BIT;
-        right[k] = LEAF_BIT | (f + cl);
+        T.perm[f + cl] = R & ~LEAF_BIT;
+        T.right[k] = LEAF_BIT | (f + cl);
     } else {
-        first[R] = f + cl;
+        T.first[R] = f + cl;
     }
-    last[k] = f + count[k] - 1u;
+    T.last[k] = f + T.count[k] - 1u;
+}
+
+__global__ void k_ploc_layout(uint32_t lo, uint32_t hi, PlocTree T) {
+    const uint32_t k = lo + blockIdx.x * blockDim.x + threadIdx.x;
+    if (k <= hi) ploc_layout_node(T, k);
+}
+
+// The last rounds (m <= PLOC_TAIL clusters) by one block, the clusters in shared memory, by the
+// same rules as the kernels above; then the layout of these rounds' nodes, which are the top
+// of the tree.  status: 1 when one cluster is left, 0 if a round merged nothing.  A round costs
+// a few microseconds here, against about 30 as four launches and a read-back.
+constexpr size_t PLOC_TAIL_SMEM = (size_t)PLOC_TAIL * (6 * sizeof(float) + 4 * sizeof(uint32_t)) + 64 * sizeof(uint32_t);
+
+__global__ void __launch_bounds__(PLOC_TAIL_THREADS) k_ploc_tail(Clusters c, uint32_t m, uint32_t merged, uint32_t n,
+                                                                 PlocTree T, DpArrays D, uint32_t* status) {
+    extern __shared__ float sm[];
+    constexpr int TH = (int)PLOC_TAIL_THREADS, CAP = (int)PLOC_TAIL;
+    float* box[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) box[a] = sm + a * CAP;
+    uint32_t* ref = reinterpret_cast<uint32_t*>(sm + 6 * CAP);
+    uint32_t* cnt = ref + CAP;
+    uint32_t* nn = cnt + CAP;
+    uint32_t* rounds = nn + CAP;            // merges before each round (at most m - 1 rounds)
+    uint32_t* wsum = rounds + CAP;          // 2 x 32 warp totals
+    const int t = (int)threadIdx.x, lane = t & 31, warp = t >> 5;
+    for (int i = t; i < (int)m; i += TH) {
+        const float4 lo = c.lo[i], hi = c.hi[i];
+        box[0][i] = lo.x; box[1][i] = lo.y; box[2][i] = lo.z;
+        box[3][i] = hi.x; box[4][i] = hi.y; box[5][i] = hi.z;
+        ref[i] = c.ref[i];
+        cnt[i] = c.cnt[i];
+    }
+    __syncthreads();
+    auto lo_of = [&](int i) { return mk3(box[0][i], box[1][i], box[2][i]); };
+    auto hi_of = [&](int i) { return mk3(box[3][i], box[4][i], box[5][i]); };
+    uint32_t n_rounds = 0;
+    bool stuck = false;
+    while (m > 1u && !stuck) {
+        for (int i = t; i < (int)m; i += TH) {
+            const float3 alo = lo_of(i), ahi = hi_of(i);
+            float best = __int_as_float(0x7f800000);
+            int bj = -1;
+            const int j0 = max(i - PLOC_R, 0), j1 = min(i + PLOC_R, (int)m - 1);
+            for (int j = j0; j <= j1; ++j) {
+                if (j == i) continue;
+                const float3 blo = lo_of(j), bhi = hi_of(j);
+                const float a = half_area3(mk3(fminf(alo.x, blo.x), fminf(alo.y, blo.y), fminf(alo.z, blo.z)),
+                                           mk3(fmaxf(ahi.x, bhi.x), fmaxf(ahi.y, bhi.y), fmaxf(ahi.z, bhi.z)));
+                if (a < best) { best = a; bj = j; }
+            }
+            nn[i] = (uint32_t)bj;
+        }
+        __syncthreads();
+        // this thread's clusters t and t + TH: survives (1), merges (1 << 16); prefix over both halves
+        uint32_t f[2], x[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t v = ploc_flag(nn, m, (uint32_t)(t + h * TH));
+            f[h] = x[h] = (uint32_t)(v & 1ull) | ((uint32_t)(v >> 32) << 16);
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t y = __shfl_up_sync(0xffffffffu, x[h], off);
+                if (lane >= off) x[h] += y;
+            }
+            if (lane == 31) wsum[32 * h + warp] = x[h];
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // inclusive scan of the 64 warp totals, first half then second
+            uint32_t a = wsum[lane], b = wsum[32 + lane];
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t ya = __shfl_up_sync(0xffffffffu, a, off), yb = __shfl_up_sync(0xffffffffu, b, off);
+                if (lane >= off) { a += ya; b += yb; }
+            }
+            b += __shfl_sync(0xffffffffu, a, 31);
+            wsum[lane] = a;
+            wsum[32 + lane] = b;
+        }
+        __syncthreads();
+        const uint32_t total = wsum[63];
+        float3 nlo[2], nhi[2];
+        uint32_t nref[2], ncnt[2], pos[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int w = 32 * h + warp, i = t + h * TH;
+            if (f[h] == 0u) continue;
+            const uint32_t pre = (w > 0 ? wsum[w - 1] : 0u) + x[h] - f[h];
+            pos[h] = pre & 0xffffu;
+            nlo[h] = lo_of(i);
+            nhi[h] = hi_of(i);
+            nref[h] = ref[i];
+            ncnt[h] = cnt[i];
+            if (f[h] >> 16) {
+                const int j = (int)nn[i];
+                const float3 l1 = lo_of(j), h1 = hi_of(j);
+                const float la = half_area_box(nlo[h], nhi[h]), ra = half_area_box(l1, h1);
+                const uint32_t node = n - 2u - (merged + (pre >> 16));
+                nlo[h] = mk3(fminf(nlo[h].x, l1.x), fminf(nlo[h].y, l1.y), fminf(nlo[h].z, l1.z));
+                nhi[h] = mk3(fmaxf(nhi[h].x, h1.x), fmaxf(nhi[h].y, h1.y), fmaxf(nhi[h].z, h1.z));
+                ncnt[h] += cnt[j];
+                T.left[node] = nref[h];
+                T.right[node] = ref[j];
+                T.count[node] = ncnt[h];
+                T.blo[node] = make_float4(nlo[h].x, nlo[h].y, nlo[h].z, 0.0f);
+                T.bhi[node] = make_float4(nhi[h].x, nhi[h].y, nhi[h].z, 0.0f);
+                if (D.cost) dp_node(D, node, nref[h], la, ref[j], ra, ncnt[h], half_area_box(nlo[h], nhi[h]));
+                nref[h] = node;
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (f[h] == 0u) continue;
+            const uint32_t q = pos[h];
+            box[0][q] = nlo[h].x; box[1][q] = nlo[h].y; box[2][q] = nlo[h].z;
+            box[3][q] = nhi[h].x; box[4][q] = nhi[h].y; box[5][q] = nhi[h].z;
+            ref[q] = nref[h];
+            cnt[q] = ncnt[h];
+        }
+        if (t == 0) rounds[n_rounds] = merged;
+        ++n_rounds;
+        stuck = (total >> 16) == 0u;
+        m -= total >> 16;
+        merged += total >> 16;
+        __syncthreads();
+    }
+    if (t == 0) *status = stuck ? 0u : 1u;
+    if (stuck) return;
+    if (t == 0) T.first[0] = 0u;
+    __syncthreads();
+    for (uint32_t r = n_rounds; r-- > 0;) {
+        const uint32_t lo = n - 1u - (r + 1u < n_rounds ? rounds[r + 1u] : n - 1u), hi = n - 2u - rounds[r];
+        for (uint32_t k = lo + (uint32_t)t; k <= hi; k += TH) ploc_layout_node(T, k);
+        __syncthreads();
+    }
 }
 
 // ------------------------------------------------------------------ collapse to wide nodes
@@ -537,9 +701,7 @@ __device__ __forceinline__ uint32_t pack_bytes(const uint32_t* q, int off) {
     return q[off] | (q[off + 1] << 8) | (q[off + 2] << 16) | (q[off + 3] << 24);
 }
 
-__global__ void k_collapse(CollapseCtx C, uint32_t qbeg, uint32_t qend) {
-    const uint32_t ti = qbeg + blockIdx.x * blockDim.x + threadIdx.x;
-    if (ti >= qend) return;
+__device__ __forceinline__ void collapse_task(const CollapseCtx& C, uint32_t ti) {
     const BinTree& T = C.T;
     const uint32_t root_ref = C.task_ref[ti];
     const uint32_t wnode = C.task_node[ti];
@@ -668,6 +830,17 @@ __global__ void k_collapse(CollapseCtx C, uint32_t qbeg, uint32_t qend) {
     o[4] = make_uint4(pack_bytes(qhi[1], 0), pack_bytes(qhi[1], 4), pack_bytes(qhi[2], 0), pack_bytes(qhi[2], 4));
 }
 
+// one level of the wide tree: the tasks levels[l] .. levels[l + 1] - 1 of the queue (a ring of 8
+// level starts); they append the next level's
+__global__ void __launch_bounds__(128) k_collapse(CollapseCtx C, const uint32_t* levels, uint32_t l) {
+    const uint32_t qbeg = levels[l & 7u], qend = levels[(l + 1u) & 7u];
+    for (uint32_t ti = qbeg + blockIdx.x * blockDim.x + threadIdx.x; ti < qend; ti += gridDim.x * blockDim.x)
+        collapse_task(C, ti);
+}
+__global__ void k_collapse_next(const uint32_t* counters, uint32_t* levels, uint32_t l) {
+    levels[(l + 2u) & 7u] = counters[2];
+}
+
 template <typename T>
 static cudaError_t dalloc(T** p, size_t n) {
     return cudaMalloc((void**)p, std::max<size_t>(n, 1) * sizeof(T));
@@ -678,20 +851,32 @@ pt_status pt_build_bvh_impl(pt_scene* s, uint32_t leaf_size, uint32_t builder, u
     const uint32_t n = s->n_tris;
     if (s->d_nodes) { cudaFree(s->d_nodes); s->d_nodes = nullptr; }
     if (s->d_tris) { cudaFree(s->d_tris); s->d_tris = nullptr; }
-    uint64_t *k0 = nullptr, *k1 = nullptr;
-    uint32_t *v0 = nullptr, *v1 = nullptr, *hist = nullptr, *cb = nullptr;
-    uint32_t *left = nullptr, *right = nullptr, *pint = nullptr, *pleaf = nullptr, *first = nullptr, *last = nullptr;
-    uint32_t *flags = nullptr, *tref = nullptr, *tnode = nullptr, *counters = nullptr;
-    float4 *blo = nullptr, *bhi = nullptr, *clo = nullptr, *chi = nullptr;
-    float* dpc = nullptr;
-    uint32_t* dpd = nullptr;
+    // all scratch in one allocation (about 30 separate ones and their frees cost more than the
+    // kernels of a small build)
     const uint32_t nblocks = (n + RS_TILE - 1) / RS_TILE;
+    const bool ploc = builder == PT_BVH_PLOC;
+    size_t used = 0;
+    auto reserve = [&](size_t bytes) {
+        const size_t at = used;
+        used += (std::max<size_t>(bytes, 1) + 255) & ~(size_t)255;
+        return at;
+    };
+    const size_t u32n = (size_t)n * sizeof(uint32_t), f4n = (size_t)n * sizeof(float4);
+    const size_t o_k0 = reserve(2 * u32n), o_k1 = reserve(2 * u32n), o_v0 = reserve(u32n), o_v1 = reserve(u32n);
+    const size_t o_hist = reserve((size_t)257 * nblocks * sizeof(uint32_t)), o_total = reserve(256 * sizeof(uint32_t));
+    const size_t o_cb = reserve(8 * sizeof(uint32_t));
+    const size_t o_left = reserve(u32n), o_right = reserve(u32n), o_pint = reserve(u32n), o_pleaf = reserve(u32n);
+    const size_t o_first = reserve(u32n), o_last = reserve(u32n), o_flags = reserve(u32n);
+    const size_t o_tref = reserve(u32n + 4), o_tnode = reserve(u32n + 4);
+    const size_t o_counters = reserve(16 * sizeof(uint32_t)), o_state = reserve(8 * sizeof(PlocState));
+    const size_t o_blo = reserve(f4n), o_bhi = reserve(f4n);
+    const size_t o_clo = reserve(ploc ? 2 * f4n : 0), o_chi = reserve(ploc ? 2 * f4n : 0);
+    const bool optimal = collapse == PT_COLLAPSE_OPTIMAL;
+    const size_t o_dpc = reserve(optimal ? (size_t)8 * n * sizeof(float) : 0), o_dpd = reserve(optimal ? u32n : 0);
+    unsigned char* scratch = nullptr;
     pt_status status = PT_OK;
     auto cleanup = [&]() {
-        void* ps[] = {k0,    k1,    v0,    v1,    hist,  cb,       left, right, pint, pleaf, first,
-                      last,  flags, tref,  tnode, counters, blo,  bhi,   clo,  chi,  dpc,   dpd};
-        for (void* q : ps)
-            if (q) cudaFree(q);
+        if (scratch) cudaFree(scratch);
     };
 #define BTRY(call)                                                                           \
     do {                                                                                     \
@@ -702,19 +887,21 @@ pt_status pt_build_bvh_impl(pt_scene* s, uint32_t leaf_size, uint32_t builder, u
             return e_ == cudaErrorMemoryAllocation ? PT_ERR_OOM : PT_ERR_CUDA;               \
         }                                                                                    \
     } while (0)
-    BTRY(dalloc(&k0, n)); BTRY(dalloc(&k1, n)); BTRY(dalloc(&v0, n)); BTRY(dalloc(&v1, n));
-    BTRY(dalloc(&hist, (size_t)256 * nblocks)); BTRY(dalloc(&cb, 8));
-    BTRY(dalloc(&left, n)); BTRY(dalloc(&right, n)); BTRY(dalloc(&pint, n)); BTRY(dalloc(&pleaf, n));
-    BTRY(dalloc(&first, n)); BTRY(dalloc(&last, n)); BTRY(dalloc(&flags, n));
-    BTRY(dalloc(&tref, n + 1)); BTRY(dalloc(&tnode, n + 1)); BTRY(dalloc(&counters, 4));
-    BTRY(dalloc(&blo, n)); BTRY(dalloc(&bhi, n));
-    if (builder == PT_BVH_PLOC) { BTRY(dalloc(&clo, (size_t)2 * n)); BTRY(dalloc(&chi, (size_t)2 * n)); }
+    BTRY(dalloc(&scratch, used));
+    auto u32 = [&](size_t o) { return reinterpret_cast<uint32_t*>(scratch + o); };
+    auto f4 = [&](size_t o) { return reinterpret_cast<float4*>(scratch + o); };
+    uint64_t *k0 = reinterpret_cast<uint64_t*>(scratch + o_k0), *k1 = reinterpret_cast<uint64_t*>(scratch + o_k1);
+    uint32_t *v0 = u32(o_v0), *v1 = u32(o_v1), *hist = u32(o_hist), *total = u32(o_total), *cb = u32(o_cb);
+    uint32_t *left = u32(o_left), *right = u32(o_right), *pint = u32(o_pint), *pleaf = u32(o_pleaf);
+    uint32_t *first = u32(o_first), *last = u32(o_last), *flags = u32(o_flags);
+    uint32_t *tref = u32(o_tref), *tnode = u32(o_tnode), *counters = u32(o_counters);
+    uint32_t* levels = counters + 8;
+    PlocState* state = reinterpret_cast<PlocState*>(scratch + o_state);
+    float4 *blo = f4(o_blo), *bhi = f4(o_bhi), *clo = f4(o_clo), *chi = f4(o_chi);
     DpArrays D{nullptr, nullptr, leaf_size, tri_cost, box_cost, max_width};
-    if (collapse == PT_COLLAPSE_OPTIMAL) {
-        BTRY(dalloc(&dpc, (size_t)8 * n));
-        BTRY(dalloc(&dpd, n));
-        D.cost = dpc;
-        D.dec = dpd;
+    if (optimal) {
+        D.cost = reinterpret_cast<float*>(scratch + o_dpc);
+        D.dec = u32(o_dpd);
     }
     BTRY(dalloc(&s->d_nodes, (size_t)5 * (n + 1)));
     BTRY(dalloc(&s->d_tris, (size_t)3 * n));
@@ -722,14 +909,14 @@ pt_status pt_build_bvh_impl(pt_scene* s, uint32_t leaf_size, uint32_t builder, u
     const uint32_t cbinit[6] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u};
     BTRY(cudaMemcpyAsync(cb, cbinit, sizeof(cbinit), cudaMemcpyHostToDevice, st));
     const uint32_t g = (n + 255) / 256;
-    PT_LAUNCH(k_centroid_bounds, g, 256, 0, st, s->d_tris_raw, n, cb);
+    PT_LAUNCH(k_centroid_bounds, std::min<uint32_t>(g, (uint32_t)pt_num_sms() * 8u), 256, 0, st, s->d_tris_raw, n, cb);
     PT_LAUNCH(k_morton, g, 256, 0, st, s->d_tris_raw, n, cb, k0, v0);
     s->launches += 2;
     for (int pass = 0; pass < 8; ++pass) {
         const int shift = 8 * pass;
         PT_LAUNCH(k_rs_hist, nblocks, RS_THREADS, 0, st, k0, n, shift, hist, nblocks);
-        PT_LAUNCH(k_rs_scan, 1, 1024, 0, st, hist, 256u * nblocks);
-        PT_LAUNCH(k_rs_scatter, nblocks, RS_THREADS, 0, st, k0, v0, k1, v1, n, shift, hist, nblocks);
+        PT_LAUNCH(k_rs_scan, 256, 256, 0, st, hist, nblocks, total);
+        PT_LAUNCH(k_rs_scatter, nblocks, RS_THREADS, 0, st, k0, v0, k1, v1, n, shift, hist, total, nblocks);
         std::swap(k0, k1);
         std::swap(v0, v1);
         s->launches += 3;
@@ -751,34 +938,57 @@ pt_status pt_build_bvh_impl(pt_scene* s, uint32_t leaf_size, uint32_t builder, u
         uint64_t* bsum = reinterpret_cast<uint64_t*>(hist);
         PT_LAUNCH(k_ploc_init, g, 256, 0, st, s->d_tris_raw, v0, n, ca);
         s->launches++;
-        std::vector<std::pair<uint32_t, uint32_t>> rounds;
-        uint32_t m = n, merged = 0;
-        while (m > 1) {
-            const uint32_t nb = (m + PLOC_SCAN_TILE - 1) / PLOC_SCAN_TILE;
-            PT_LAUNCH(k_ploc_nn, (m + PLOC_THREADS - 1) / PLOC_THREADS, PLOC_THREADS, 0, st, ca, m, pint);
-            PT_LAUNCH(k_ploc_scan, nb, PLOC_THREADS, 0, st, pint, m, pre, bsum);
-            PT_LAUNCH(k_ploc_scan_top, 1, 1024, 0, st, bsum, nb);
-            PT_LAUNCH(k_ploc_compact, (m + 255) / 256, 256, 0, st, ca, cb2, pint, m, pre, bsum, n, merged, left,
-                      right, pleaf, blo, bhi, D);
-            s->launches += 4;
-            uint64_t total = 0;
-            BTRY(cudaMemcpyAsync(&total, bsum + nb, sizeof(total), cudaMemcpyDeviceToHost, st));
-            BTRY(cudaStreamSynchronize(st));
-            const uint32_t merges = (uint32_t)(total >> 32), m_new = (uint32_t)(total & 0xffffffffull);
-            if (merges == 0 || m_new != m - merges || merged + merges > n - 1) {
-                pt_set_error("PLOC clustering made no progress");
-                cleanup();
-                return PT_ERR_CUDA;
+        const PlocTree PT{left, right, pleaf, first, last, v1, blo, bhi};
+        std::vector<PlocState> rounds;      // state before each round outside the tail
+        PlocState now{n, 0u};
+        BTRY(cudaMemcpyAsync(state, &now, sizeof(now), cudaMemcpyHostToDevice, st));
+        uint32_t r = 0;
+        while (now.m > PLOC_TAIL) {
+            // grids for the clusters known to be left; later rounds of the batch have fewer
+            const uint32_t m = now.m, nb = (m + PLOC_SCAN_TILE - 1) / PLOC_SCAN_TILE;
+            Clusters x = ca, y = cb2;
+            for (uint32_t k = 0; k < PLOC_BATCH; ++k) {
+                const PlocState* cur = state + ((r + k) & 7u);
+                PT_LAUNCH(k_ploc_nn, (m + PLOC_THREADS - 1) / PLOC_THREADS, PLOC_THREADS, 0, st, x, cur, pint);
+                PT_LAUNCH(k_ploc_scan, nb, PLOC_THREADS, 0, st, pint, cur, pre, bsum);
+                PT_LAUNCH(k_ploc_scan_top, 1, 1024, 0, st, bsum, cur, state + ((r + k + 1u) & 7u));
+                PT_LAUNCH(k_ploc_compact, (m + 255) / 256, 256, 0, st, x, y, pint, cur, pre, bsum, n, left, right,
+                          pleaf, blo, bhi, D);
+                s->launches += 4;
+                std::swap(x, y);
             }
-            rounds.emplace_back(n - 1 - merged - merges, n - 2 - merged);
-            merged += merges;
-            m = m_new;
-            std::swap(ca, cb2);
+            PlocState ring[8];
+            BTRY(cudaMemcpyAsync(ring, state, sizeof(ring), cudaMemcpyDeviceToHost, st));
+            BTRY(cudaStreamSynchronize(st));
+            for (uint32_t k = 0; k < PLOC_BATCH && now.m > PLOC_TAIL; ++k) {
+                const PlocState nx = ring[(r + k + 1u) & 7u];
+                if (nx.m >= now.m || nx.m == 0u || nx.merged + nx.m != n) {
+                    pt_set_error("PLOC clustering made no progress");
+                    cleanup();
+                    return PT_ERR_CUDA;
+                }
+                rounds.push_back(now);
+                now = nx;
+                std::swap(ca, cb2);
+            }
+            r += PLOC_BATCH;
         }
-        BTRY(cudaMemsetAsync(first, 0, sizeof(uint32_t), st));
-        for (size_t r = rounds.size(); r-- > 0;) {
-            const uint32_t lo = rounds[r].first, hi = rounds[r].second;
-            PT_LAUNCH(k_ploc_layout, (hi - lo + 1 + 255) / 256, 256, 0, st, lo, hi, left, right, pleaf, first, last, v1);
+        static_assert(PLOC_TAIL <= 2 * PLOC_TAIL_THREADS && PLOC_BATCH <= 4, "two clusters a thread; the ring holds a batch");
+        BTRY(cudaFuncSetAttribute(k_ploc_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PLOC_TAIL_SMEM));
+        PT_LAUNCH(k_ploc_tail, 1, PLOC_TAIL_THREADS, PLOC_TAIL_SMEM, st, ca, now.m, now.merged, n, PT, D, counters);
+        s->launches++;
+        uint32_t done = 0;
+        BTRY(cudaMemcpyAsync(&done, counters, sizeof(done), cudaMemcpyDeviceToHost, st));
+        BTRY(cudaStreamSynchronize(st));
+        if (!done) {
+            pt_set_error("PLOC clustering made no progress");
+            cleanup();
+            return PT_ERR_CUDA;
+        }
+        for (size_t q = rounds.size(); q-- > 0;) {
+            const uint32_t merged_after = q + 1 < rounds.size() ? rounds[q + 1].merged : now.merged;
+            const uint32_t lo = n - 1u - merged_after, hi = n - 2u - rounds[q].merged;
+            PT_LAUNCH(k_ploc_layout, (hi - lo + 1 + 255) / 256, 256, 0, st, lo, hi, PT);
             s->launches++;
         }
         T.perm = v1;
@@ -801,17 +1011,27 @@ pt_status pt_build_bvh_impl(pt_scene* s, uint32_t leaf_size, uint32_t builder, u
     C.out_tris = s->d_tris;
     C.in_tris = s->d_tris_raw;
     C.dp = D;
-    uint32_t qbeg = 0, qend = 1, depth = 0;
-    uint32_t host_counters[4] = {0, 0, 0, 0};
-    while (qbeg < qend) {
-        const uint32_t cnt = qend - qbeg;
-        PT_LAUNCH(k_collapse, (cnt + 127) / 128, 128, 0, st, C, qbeg, qend);
-        s->launches++;
+    // the levels run without the host, four between read-backs of the queue: a level has at most
+    // max_width times the tasks of the one before it
+    const uint32_t level_init[8] = {0u, 1u, 0u, 0u, 0u, 0u, 0u, 0u};
+    BTRY(cudaMemcpyAsync(levels, level_init, sizeof(level_init), cudaMemcpyHostToDevice, st));
+    uint32_t depth = 0, l = 0;
+    uint64_t width_ub = 1;
+    uint32_t host_counters[16] = {0};
+    for (bool more = true; more;) {
+        for (uint32_t k = 0; k < 4; ++k, ++l) {
+            const uint32_t grid = (uint32_t)std::min<uint64_t>((width_ub + 127) / 128, (uint64_t)pt_num_sms() * 16);
+            PT_LAUNCH(k_collapse, grid, 128, 0, st, C, levels, l);
+            PT_LAUNCH(k_collapse_next, 1, 1, 0, st, counters, levels, l);
+            s->launches += 2;
+            width_ub = std::min<uint64_t>(width_ub * max_width, n);
+        }
         BTRY(cudaMemcpyAsync(host_counters, counters, sizeof(host_counters), cudaMemcpyDeviceToHost, st));
         BTRY(cudaStreamSynchronize(st));
-        ++depth;
-        qbeg = qend;
-        qend = host_counters[2];
+        for (uint32_t k = l - 4; k < l && more; ++k) {
+            if (host_counters[8 + (k & 7u)] < host_counters[8 + ((k + 1u) & 7u)]) ++depth;
+            else more = false;
+        }
         if (depth > 200) { pt_set_error("BVH collapse did not terminate"); status = PT_ERR_CUDA; break; }
     }
     BTRY(cudaGetLastError());

@@ -207,5 +207,36 @@ inline DCam to_dcam(const pt_camera& c) {
     return d;
 }
 
+// ---- bounds of many points: floats as unsigned integers of the same order, min/max by atomics
+__device__ __forceinline__ uint32_t f2ord(float f) {
+    const uint32_t b = __float_as_uint(f);
+    return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
+}
+__device__ __forceinline__ float ord2f(uint32_t u) {
+    return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
+}
+// lo / hi of every thread of the block (at most 1024 threads, all of them) into bounds[0..2] / [3..5]
+__device__ __forceinline__ void block_bounds(float3 lo, float3 hi, uint32_t* bounds) {
+    __shared__ float part[6][32];
+    float v[6] = {lo.x, lo.y, lo.z, hi.x, hi.y, hi.z};
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            const float o = __shfl_xor_sync(0xffffffffu, v[a], off);
+            v[a] = a < 3 ? fminf(v[a], o) : fmaxf(v[a], o);
+        }
+        if ((threadIdx.x & 31u) == 0) part[a][threadIdx.x >> 5] = v[a];
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int a = (int)threadIdx.x;
+        float x = part[a][0];
+        for (uint32_t w = 1; w < (blockDim.x + 31u) >> 5; ++w) x = a < 3 ? fminf(x, part[a][w]) : fmaxf(x, part[a][w]);
+        if (a < 3) atomicMin(&bounds[a], f2ord(x));
+        else atomicMax(&bounds[a], f2ord(x));
+    }
+}
+
 // device-side material repack (runs the conversion in a kernel)
 struct RawMat { float v[PT_OPENPBR_FLOATS]; };
