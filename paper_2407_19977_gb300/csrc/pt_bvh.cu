@@ -697,145 +697,174 @@ __device__ __forceinline__ float area(const Box& b) {
     return dx * dy + dy * dz + dz * dx;
 }
 
-__device__ __forceinline__ uint32_t pack_bytes(const uint32_t* q, int off) {
-    return q[off] | (q[off + 1] << 8) | (q[off + 2] << 16) | (q[off + 3] << 24);
-}
-
-__device__ __forceinline__ void collapse_task(const CollapseCtx& C, uint32_t ti) {
+// One wide node by a group of 8 lanes, lane = child slot: unfolding, boxes, quantisation and the
+// copies of the leaves' triangles are chains of dependent loads and divisions, so a thread per
+// node took 75 us a level, even a level of one node (17 levels, 1.28 ms of a 1.07M-triangle
+// build); side by side a level takes 21 (20 launches, 0.42 ms).
+__device__ __forceinline__ void collapse_task(const CollapseCtx& C, uint32_t ti, uint32_t gl, uint32_t gm, uint32_t gbase) {
     const BinTree& T = C.T;
     const uint32_t root_ref = C.task_ref[ti];
     const uint32_t wnode = C.task_node[ti];
-    uint32_t ch[8];
-    Box cb[8];
-    int nc = 0;
+    constexpr uint32_t NONE = 0xffffffffu;     // an empty slot
+    uint32_t ref = NONE;
     if ((root_ref & LEAF_BIT) || ref_count(T, root_ref) <= C.leaf_size) {
-        ch[0] = root_ref;
-        cb[0] = ref_box(T, root_ref);
-        nc = 1;
+        if (gl == 0) ref = root_ref;
     } else if (C.dp.cost) {
-        // unfold the choices: the root's split, then each part's split of its slot budget
-        uint32_t sref[8], sj[8];
-        int sp = 0;
-        const uint32_t d0 = C.dp.dec[root_ref];
-        const uint32_t j0 = min(max(d0 & 15u, 2u), 8u);
-        const uint32_t i0 = (d0 >> (4u * (j0 - 1u))) & 15u;
-        sref[sp] = T.right[root_ref]; sj[sp++] = j0 - i0;
-        sref[sp] = T.left[root_ref]; sj[sp++] = i0;
-        while (sp > 0) {
-            const uint32_t r = sref[--sp], j = sj[sp];
-            const uint32_t i = (r & LEAF_BIT) || j < 2u || j > 8u ? 0u : (C.dp.dec[r] >> (4u * (j - 1u))) & 15u;
-            if (i == 0u || i >= j || nc + sp + 2 > 8) {   // one slot (valid choices never need the guards)
-                ch[nc] = r;
-                cb[nc] = ref_box(T, r);
-                ++nc;
+        // unfold the choices side by side: a part with a budget of j slots starts at lane `gl`
+        // and owns j lanes; its left child keeps the first i of them, the right child the rest
+        uint32_t j = 0;
+        if (gl == 0) {
+            ref = root_ref;
+            j = min(max(C.dp.dec[root_ref] & 15u, 2u), 8u);
+        }
+        for (;;) {
+            uint32_t i = 0, right = NONE, rj = 0;
+            if (ref != NONE && !(ref & LEAF_BIT) && j >= 2u) i = (C.dp.dec[ref] >> (4u * (j - 1u))) & 15u;
+            const bool split = i > 0u && i < j;
+            if (split) {
+                right = T.right[ref];
+                ref = T.left[ref];
+                rj = j - i;
+                j = i;
             } else {
-                sref[sp] = T.right[r]; sj[sp++] = j - i;
-                sref[sp] = T.left[r]; sj[sp++] = i;
+                j = min(j, 1u);      // one slot
+            }
+            const uint32_t splits = (__ballot_sync(gm, split) >> gbase) & 0xffu;
+            if (splits == 0u) break;
+            // the part whose right child starts at this lane, if any
+            const uint32_t target = split ? gl + i : 8u;
+#pragma unroll
+            for (uint32_t q = 0; q < 8; ++q) {
+                const uint32_t tq = __shfl_sync(gm, target, q, 8), rq = __shfl_sync(gm, right, q, 8),
+                               jq = __shfl_sync(gm, rj, q, 8);
+                if (tq == gl) { ref = rq; j = jq; }
             }
         }
     } else {
+        // greedy, largest child first; every lane of the group makes the same choices
+        uint32_t ch[8];
+        float ca[8];
         ch[0] = T.left[root_ref];
         ch[1] = T.right[root_ref];
-        cb[0] = ref_box(T, ch[0]);
-        cb[1] = ref_box(T, ch[1]);
-        nc = 2;
+        int nc = 2;
+        for (int k = 0; k < 2; ++k) ca[k] = area(ref_box(T, ch[k]));
         while (nc < (int)C.width) {
             int best = -1;
             float best_a = -1.0f;
-            for (int j = 0; j < nc; ++j) {
-                if ((ch[j] & LEAF_BIT) || ref_count(T, ch[j]) <= C.leaf_size) continue;
-                const float a = area(cb[j]);
-                if (a > best_a) { best_a = a; best = j; }
+            for (int k = 0; k < nc; ++k) {
+                if ((ch[k] & LEAF_BIT) || ref_count(T, ch[k]) <= C.leaf_size) continue;
+                if (ca[k] > best_a) { best_a = ca[k]; best = k; }
             }
             if (best < 0) break;
             const uint32_t r = ch[best];
             ch[best] = T.left[r];
-            cb[best] = ref_box(T, ch[best]);
+            ca[best] = area(ref_box(T, ch[best]));
             ch[nc] = T.right[r];
-            cb[nc] = ref_box(T, ch[nc]);
+            ca[nc] = area(ref_box(T, ch[nc]));
             ++nc;
         }
+        if ((int)gl < nc) ref = ch[gl];
     }
-    uint32_t n_int = 0, n_leaf_tris = 0;
-    for (int j = 0; j < nc; ++j) {
-        const uint32_t c = ref_count(T, ch[j]);
-        if (c > C.leaf_size) ++n_int; else n_leaf_tris += c;
+    const bool used = ref != NONE;
+    const float inf = __int_as_float(0x7f800000);
+    Box cb;
+    cb.lo = splat3(inf);
+    cb.hi = splat3(-inf);
+    uint32_t c = 0;
+    if (used) {
+        cb = ref_box(T, ref);
+        c = ref_count(T, ref);
     }
-    const uint32_t child_base = n_int ? atomicAdd(&C.counters[0], n_int) : 0u;
-    const uint32_t tri_base = n_leaf_tris ? atomicAdd(&C.counters[1], n_leaf_tris) : 0u;
-    const uint32_t qpos = n_int ? atomicAdd(&C.counters[2], n_int) : 0u;
+    const bool inner = c > C.leaf_size;
+    const uint32_t imask = (__ballot_sync(gm, inner) >> gbase) & 0xffu;
+    const uint32_t n_int = __popc(imask), rank = __popc(imask & ((1u << gl) - 1u));
+    // leaf triangles before this slot's
+    const uint32_t lc = inner ? 0u : c;
+    uint32_t incl = lc;
+#pragma unroll
+    for (uint32_t d = 1; d < 8; d <<= 1) {
+        const uint32_t y = __shfl_up_sync(gm, incl, d, 8);
+        if (gl >= d) incl += y;
+    }
+    const uint32_t toff = incl - lc, n_leaf_tris = __shfl_sync(gm, incl, 7, 8);
+    // lanes 0..2 reserve the node's children, triangles and queue entries
+    uint32_t base = 0;
+    if (gl < 3) {
+        const uint32_t want = gl == 1 ? n_leaf_tris : n_int;
+        if (want) base = atomicAdd(&C.counters[gl], want);
+    }
+    const uint32_t child_base = __shfl_sync(gm, base, 0, 8), tri_base = __shfl_sync(gm, base, 1, 8),
+                   qpos = __shfl_sync(gm, base, 2, 8);
     // node box and quantisation frame
-    Box nb = cb[0];
-    for (int j = 1; j < nc; ++j) nb = box_union(nb, cb[j]);
+    Box nb = cb;
+#pragma unroll
+    for (uint32_t d = 1; d < 8; d <<= 1) {
+        Box o;
+        o.lo = mk3(__shfl_xor_sync(gm, nb.lo.x, d, 8), __shfl_xor_sync(gm, nb.lo.y, d, 8), __shfl_xor_sync(gm, nb.lo.z, d, 8));
+        o.hi = mk3(__shfl_xor_sync(gm, nb.hi.x, d, 8), __shfl_xor_sync(gm, nb.hi.y, d, 8), __shfl_xor_sync(gm, nb.hi.z, d, 8));
+        nb = box_union(nb, o);
+    }
     const float3 p = nb.lo;
-    float ext[3] = {nb.hi.x - nb.lo.x, nb.hi.y - nb.lo.y, nb.hi.z - nb.lo.z};
-    const float emax = fmaxf(ext[0], fmaxf(ext[1], ext[2]));
+    const float emax = fmaxf(nb.hi.x - nb.lo.x, fmaxf(nb.hi.y - nb.lo.y, nb.hi.z - nb.lo.z));
     uint32_t ebias[3];
-    float scale[3];
+    unsigned char* node = reinterpret_cast<unsigned char*>(C.nodes + 5u * wnode);
+#pragma unroll
     for (int a = 0; a < 3; ++a) {
-        const float e = fmaxf(fmaxf(ext[a], emax * 1e-6f), 1e-30f);
+        const float pa = comp3(p, a);
+        const float e = fmaxf(fmaxf(comp3(nb.hi, a) - pa, emax * 1e-6f), 1e-30f);
         int ex;
         frexpf(e / 255.0f, &ex);
-        int b = min(max(ex + 127, 1), 254);
-        float sc = __uint_as_float((uint32_t)b << 23);
-        while (b < 254 && fmaf(255.0f, sc, comp3(p, a)) < comp3(nb.hi, a)) { ++b; sc = __uint_as_float((uint32_t)b << 23); }
-        ebias[a] = (uint32_t)b;
-        scale[a] = sc;
-    }
-    uint32_t qlo[3][8], qhi[3][8], meta[8];
-    uint32_t imask = 0, rank = 0, toff = 0;
-    for (int j = 0; j < 8; ++j) {
-        meta[j] = 0;
-        for (int a = 0; a < 3; ++a) { qlo[a][j] = 0; qhi[a][j] = 0; }
-    }
-    for (int j = 0; j < nc; ++j) {
-        for (int a = 0; a < 3; ++a) {
-            const float pa = comp3(p, a), sc = scale[a];
-            const float lo = comp3(cb[j].lo, a), hi = comp3(cb[j].hi, a);
+        int bb = min(max(ex + 127, 1), 254);
+        float sc = __uint_as_float((uint32_t)bb << 23);
+        while (bb < 254 && fmaf(255.0f, sc, pa) < comp3(nb.hi, a)) { ++bb; sc = __uint_as_float((uint32_t)bb << 23); }
+        ebias[a] = (uint32_t)bb;
+        uint32_t qlo = 0, qhi = 0;
+        if (used) {
+            const float lo = comp3(cb.lo, a), hi = comp3(cb.hi, a);
             float ql = floorf(__fsub_rd(lo, pa) / sc);
             ql = fminf(fmaxf(ql, 0.0f), 255.0f);
             while (ql > 0.0f && fmaf(ql, sc, pa) > lo) ql -= 1.0f;
             float qh = ceilf(__fsub_ru(hi, pa) / sc);
             qh = fminf(fmaxf(qh, 0.0f), 255.0f);
             while (qh < 255.0f && fmaf(qh, sc, pa) < hi) qh += 1.0f;
-            qlo[a][j] = (uint32_t)ql;
-            qhi[a][j] = (uint32_t)qh;
+            qlo = (uint32_t)ql;
+            qhi = (uint32_t)qh;
         }
-        const uint32_t c = ref_count(T, ch[j]);
-        if (c > C.leaf_size) {
-            imask |= 1u << j;
-            meta[j] = 1u;
-            C.task_ref[qpos + rank] = ch[j];
-            C.task_node[qpos + rank] = child_base + rank;
-            ++rank;
-        } else {
-            meta[j] = (c << 5) | toff;
-            const uint32_t f = ref_first(T, ch[j]);
-            for (uint32_t k = 0; k < c; ++k) {
-                const uint32_t src = T.perm[f + k];
-                const uint32_t dst = tri_base + toff + k;
-                C.out_tris[3u * dst + 0] = C.in_tris[3u * src + 0];
-                C.out_tris[3u * dst + 1] = C.in_tris[3u * src + 1];
-                C.out_tris[3u * dst + 2] = C.in_tris[3u * src + 2];
-            }
-            toff += c;
+        node[32 + 8 * a + gl] = (unsigned char)qlo;
+        node[56 + 8 * a + gl] = (unsigned char)qhi;
+    }
+    node[24 + gl] = (unsigned char)(inner ? 1u : c ? (c << 5) | toff : 0u);
+    if (gl == 0) {
+        C.nodes[5u * wnode] = make_uint4(__float_as_uint(p.x), __float_as_uint(p.y), __float_as_uint(p.z),
+                                         ebias[0] | (ebias[1] << 8) | (ebias[2] << 16) | (imask << 24));
+        *reinterpret_cast<uint2*>(C.nodes + 5u * wnode + 1) = make_uint2(child_base, tri_base);
+    }
+    if (inner) {
+        C.task_ref[qpos + rank] = ref;
+        C.task_node[qpos + rank] = child_base + rank;
+    } else if (used) {
+        const uint32_t f = ref_first(T, ref);
+        uint32_t src[4];      // a leaf has at most 4 triangles
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) src[k] = k < c ? T.perm[f + k] : 0u;
+#pragma unroll
+        for (uint32_t k = 0; k < 4; ++k) {
+            if (k >= c) continue;
+            const uint32_t dst = tri_base + toff + k;
+            C.out_tris[3u * dst + 0] = C.in_tris[3u * src[k] + 0];
+            C.out_tris[3u * dst + 1] = C.in_tris[3u * src[k] + 1];
+            C.out_tris[3u * dst + 2] = C.in_tris[3u * src[k] + 2];
         }
     }
-    uint4* o = C.nodes + 5u * wnode;
-    o[0] = make_uint4(__float_as_uint(p.x), __float_as_uint(p.y), __float_as_uint(p.z),
-                      ebias[0] | (ebias[1] << 8) | (ebias[2] << 16) | (imask << 24));
-    o[1] = make_uint4(child_base, tri_base, pack_bytes(meta, 0), pack_bytes(meta, 4));
-    o[2] = make_uint4(pack_bytes(qlo[0], 0), pack_bytes(qlo[0], 4), pack_bytes(qlo[1], 0), pack_bytes(qlo[1], 4));
-    o[3] = make_uint4(pack_bytes(qlo[2], 0), pack_bytes(qlo[2], 4), pack_bytes(qhi[0], 0), pack_bytes(qhi[0], 4));
-    o[4] = make_uint4(pack_bytes(qhi[1], 0), pack_bytes(qhi[1], 4), pack_bytes(qhi[2], 0), pack_bytes(qhi[2], 4));
 }
 
 // one level of the wide tree: the tasks levels[l] .. levels[l + 1] - 1 of the queue (a ring of 8
 // level starts); they append the next level's
 __global__ void __launch_bounds__(128) k_collapse(CollapseCtx C, const uint32_t* levels, uint32_t l) {
     const uint32_t qbeg = levels[l & 7u], qend = levels[(l + 1u) & 7u];
-    for (uint32_t ti = qbeg + blockIdx.x * blockDim.x + threadIdx.x; ti < qend; ti += gridDim.x * blockDim.x)
-        collapse_task(C, ti);
+    const uint32_t gl = threadIdx.x & 7u, gbase = threadIdx.x & 24u, gm = 0xffu << gbase;
+    for (uint32_t ti = qbeg + ((blockIdx.x * blockDim.x + threadIdx.x) >> 3); ti < qend; ti += (gridDim.x * blockDim.x) >> 3)
+        collapse_task(C, ti, gl, gm, gbase);
 }
 __global__ void k_collapse_next(const uint32_t* counters, uint32_t* levels, uint32_t l) {
     levels[(l + 2u) & 7u] = counters[2];
@@ -1020,7 +1049,7 @@ pt_status pt_build_bvh_impl(pt_scene* s, uint32_t leaf_size, uint32_t builder, u
     uint32_t host_counters[16] = {0};
     for (bool more = true; more;) {
         for (uint32_t k = 0; k < 4; ++k, ++l) {
-            const uint32_t grid = (uint32_t)std::min<uint64_t>((width_ub + 127) / 128, (uint64_t)pt_num_sms() * 16);
+            const uint32_t grid = (uint32_t)std::min<uint64_t>((width_ub + 15) / 16, (uint64_t)pt_num_sms() * 16);
             PT_LAUNCH(k_collapse, grid, 128, 0, st, C, levels, l);
             PT_LAUNCH(k_collapse_next, 1, 1, 0, st, counters, levels, l);
             s->launches += 2;
