@@ -20,9 +20,14 @@ namespace {
 // ------------------------------------------------------------------ primary-hit features
 __global__ void k_features(DScene S, DCam cam, uint32_t x0, uint32_t y0, uint32_t cw, uint32_t ch, uint32_t s0,
                            uint32_t spp, uint64_t seed, float4* out) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= cw * ch) return;
-    const uint32_t px = x0 + i % cw, py = y0 + i / cw;
+    // a warp covers a compact 8 x 4 tile of the window, whose camera rays meet the same nodes, and
+    // traces with the branching loop, which suits them (1080p preview with its features: 3.42 ms
+    // with rows of 32 pixels, 3.34 in tiles, 3.28 with that loop)
+    const uint32_t tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u, tw = (cw + 7u) / 8u;
+    const uint32_t wx = (tile % tw) * 8u + (lane & 7u), wy = (tile / tw) * 4u + (lane >> 3);
+    if (wx >= cw || wy >= ch) return;
+    const uint32_t i = wy * cw + wx;
+    const uint32_t px = x0 + wx, py = y0 + wy;
     const uint32_t p = py * cam.width + px;
     float3 n_sum = splat3(0.0f), x_sum = splat3(0.0f), a_sum = splat3(0.0f);
     float hits = 0.0f;
@@ -30,7 +35,8 @@ __global__ void k_features(DScene S, DCam cam, uint32_t x0, uint32_t y0, uint32_
         float3 o, d;
         camera_ray_ps(cam, px, py, p, s0 + k, (uint32_t)seed, (uint32_t)(seed >> 32), o, d);
         HitRec h;
-        trace_closest(S, o, d, __int_as_float(0x7f800000), h);
+        TravCount cnt = {0, 0, 0};
+        trace_closest_t<false>(S, o, d, __int_as_float(0x7f800000), h, cnt);
         if (h.tri == PT_NO_HIT) continue;
         const float4 ta = __ldg(S.tris + 3u * h.tri), tb = __ldg(S.tris + 3u * h.tri + 1),
                      tc = __ldg(S.tris + 3u * h.tri + 2);
@@ -300,7 +306,8 @@ extern "C" pt_status pt_render_features(pt_scene* s, const pt_camera* camera, ui
     const uint64_t n = (uint64_t)width * height;
     if (n == 0) return PT_OK;
     PT_CHECK_ARG(n < (1ull << 31), "window too large");
-    PT_LAUNCH(k_features, (uint32_t)((n + 127) / 128), 128, 0, (cudaStream_t)cuda_stream, s->view(), to_dcam(*camera),
+    const uint64_t tiles = (uint64_t)((width + 7u) / 8u) * ((height + 3u) / 4u);
+    PT_LAUNCH(k_features, (uint32_t)((tiles + 3) / 4), 128, 0, (cudaStream_t)cuda_stream, s->view(), to_dcam(*camera),
               crop_x0, crop_y0, width, height, s0, spp, seed, reinterpret_cast<float4*>(out));
     PT_CUDA_TRY(cudaGetLastError());
     return PT_OK;
