@@ -328,7 +328,10 @@ __global__ void k_bottom_up(BinTree T, int n, const uint32_t* par_int, const uin
 // node's children have higher indices than the node.  A top-down pass over the rounds in
 // reverse then lays the triangles out in tree order, giving each subtree the contiguous
 // [first, last] range the collapse needs.
-constexpr int PLOC_R = 16;
+// 8, 16 and 32 give equally good trees (closest-hit passes of the 1080p CAD frame 2.99 / 3.03 /
+// 2.99 ms, of the glass scene 2.11 / 2.18 / 2.18) and the search grows with it: opening a
+// 1.07M-triangle model takes 5.1 / 5.5 / 5.95 ms.
+constexpr int PLOC_R = 8;
 constexpr int PLOC_THREADS = 256;
 constexpr int PLOC_SCAN_ITEMS = 4;                      // per thread of the block scan
 constexpr int PLOC_SCAN_TILE = PLOC_THREADS * PLOC_SCAN_ITEMS;
