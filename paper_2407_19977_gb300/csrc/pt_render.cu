@@ -418,22 +418,19 @@ __device__ __forceinline__ uint32_t wfm_seg_of(const WfParams& P, uint32_t id) {
     return lo;
 }
 
-// scene, depth, flags and random-number keys of path id of a merged batch wave, from its
-// segment (whose wave-local index the path carries in the w word of its radiance)
-__device__ __forceinline__ void wfm_context(const WfParams& P, uint32_t seg, uint32_t id, DScene& S, VertexRng& rng,
-                                            uint32_t& max_depth, uint32_t& flags, uint32_t& job) {
+// random-number keys of path id of a merged batch wave, from its segment (whose wave-local index
+// the path carries in the w word of its radiance); returns the job, whose scene, depth and flags
+// are read in place (a copy of the scene per lane was spilled)
+__device__ __forceinline__ uint32_t wfm_rng(const WfParams& P, uint32_t seg, uint32_t id, VertexRng& rng) {
     const WfmSeg g = P.segs[seg];
     const DJob& J = P.jobs[g.job];
-    S = J.S;
     const uint32_t local = id - g.path0;
     const uint32_t lp = g.pb + local % g.npix;
     rng.p = (J.y0 + lp / J.cw) * J.cam.width + (J.x0 + lp % J.cw);
     rng.s = J.s0 + g.i0 + local / g.npix;
     rng.k0 = (uint32_t)J.seed;
     rng.k1 = (uint32_t)(J.seed >> 32);
-    max_depth = J.max_depth;
-    flags = J.flags;
-    job = g.job;
+    return g.job;
 }
 
 constexpr uint32_t NRC_DIM_TRAIN = 10;   // uniform dimension of the training-path choice
@@ -940,8 +937,23 @@ __global__ void __launch_bounds__(128, 6) k_restir_spatial(WfParams P, uint32_t 
     }
 }
 
+// 16 bytes from global to shared memory without a register
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// One path vertex per lane in the material-sorted order.  Bound by the latency of a chain of
+// gathers (order -> ray and hit -> path state and triangle -> material -> light), with a third
+// of the issue slots busy.  The ray and hit records of a warp's next 32 paths are copied to
+// shared memory while the current ones are shaded, and the order is read one step further
+// ahead (1080p CAD step: shade passes 1.99 -> 1.89 ms).  5 blocks of 96 registers per SM; 4 of
+// 128 for the forms that spill most: many lights with reservoirs 0.57 -> 0.53 ms, merged batch
+// 14.72 -> 14.44 ms a pass, but the CAD step 1.89 -> 2.05; 6 blocks 1.97.
+constexpr int shade_blocks(bool ris, bool multi) { return ris || multi ? 4 : 5; }
+
 template <bool NRC, bool RIS, bool FUZZ = true, bool MULTI = false>
-__global__ void __launch_bounds__(128, 5) k_wf_shade(WfParams P, int in_q, int out_q, uint32_t k) {
+__global__ void __launch_bounds__(128, shade_blocks(RIS, MULTI)) k_wf_shade(WfParams P, int in_q, int out_q, uint32_t k) {
     if (P.counters[C_TAIL]) return;
     const uint32_t count = P.counters[in_q];
     const uint32_t sbase = wf_sample_base(P);
@@ -950,6 +962,16 @@ __global__ void __launch_bounds__(128, 5) k_wf_shade(WfParams P, int in_q, int o
     const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
     const uint32_t lt = (1u << lane) - 1u;
     unsigned long long rr_cnt = 0;
+    __shared__ float4 stage[3][128];
+    const uint32_t step = nwarps * 32u, t = threadIdx.x;
+    const uint32_t i0 = ((blockIdx.x * blockDim.x + t) >> 5) * 32u + lane;
+    uint32_t next_slot = i0 < count ? (P.n_keys ? P.perm[i0] : i0) : 0u;
+    if (i0 < count) {
+        cp_async16(&stage[0][t], P.ray_o[in_q] + next_slot);
+        cp_async16(&stage[1][t], P.ray_d[in_q] + next_slot);
+        cp_async16(&stage[2][t], P.hit + next_slot);
+    }
+    next_slot = i0 + step < count ? (P.n_keys ? P.perm[i0 + step] : i0 + step) : 0u;
     for (uint32_t base = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32u; base < count; base += nwarps * 32u) {
         const uint32_t i = base + lane;
         const bool valid = i < count;
@@ -960,9 +982,15 @@ __global__ void __launch_bounds__(128, 5) k_wf_shade(WfParams P, int in_q, int o
         float tag = 0.0f;   // merged batch waves: the job, carried by the appended rays
         float4 b4 = make_float4(0, 0, 0, 0);
         if (valid) {
-            const uint32_t slot = P.n_keys ? P.perm[i] : i;
-            const float4 ro = P.ray_o[in_q][slot], rd = P.ray_d[in_q][slot];
-            const float4 hh = P.hit[slot];
+            cp_async_wait_all();
+            const float4 ro = stage[0][t], rd = stage[1][t];
+            const float4 hh = stage[2][t];
+            if (i + step < count) {
+                cp_async16(&stage[0][t], P.ray_o[in_q] + next_slot);
+                cp_async16(&stage[1][t], P.ray_d[in_q] + next_slot);
+                cp_async16(&stage[2][t], P.hit + next_slot);
+                if (i + 2u * step < count) next_slot = P.n_keys ? P.perm[i + 2u * step] : i + 2u * step;
+            }
             id = __float_as_uint(rd.w);
             HitRec h;
             h.t = hh.x; h.u = hh.y; h.v = hh.z; h.tri = __float_as_uint(hh.w);
@@ -973,10 +1001,9 @@ __global__ void __launch_bounds__(128, 5) k_wf_shade(WfParams P, int in_q, int o
             ps.prev_pdf = b4.w;
             ps.L = xyz(L4);
             VertexRng rng;
-            DScene Sm;
-            uint32_t md = 0, fl = 0, job = 0;
+            uint32_t job = 0;
             if constexpr (MULTI) {
-                wfm_context(P, __float_as_uint(L4.w), id, Sm, rng, md, fl, job);
+                job = wfm_rng(P, __float_as_uint(L4.w), id, rng);
             } else {
                 const uint32_t lp = P.pb + id % P.npix;
                 rng.p = (P.y0 + lp / P.cw) * P.cam.width + (P.x0 + lp % P.cw);
@@ -988,7 +1015,8 @@ __global__ void __launch_bounds__(128, 5) k_wf_shade(WfParams P, int in_q, int o
             ShadeOut so;
             int r;
             if constexpr (MULTI) {
-                r = shade_vertex<false, FUZZ>(Sm, h, xyz(ro), xyz(rd), k, md, fl, rng, ps, so, nullptr, 0u);
+                const DJob& J = P.jobs[job];
+                r = shade_vertex<false, FUZZ>(J.S, h, xyz(ro), xyz(rd), k, J.max_depth, J.flags, rng, ps, so, nullptr, 0u);
             } else if (NRC) {
                 NrcHook hook;
                 hook.P = &P;
@@ -1297,10 +1325,9 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
         ps.prev_pdf = b4.w;
         ps.L = xyz(L4);
         VertexRng rng;
-        DScene Sm;
-        uint32_t md = 0, fl = 0, job = 0;
+        uint32_t job = 0;
         if constexpr (MULTI) {
-            wfm_context(P, __float_as_uint(L4.w), id, Sm, rng, md, fl, job);
+            job = wfm_rng(P, __float_as_uint(L4.w), id, rng);
         } else {
             const uint32_t lp = P.pb + id % P.npix;
             rng.p = (P.y0 + lp / P.cw) * P.cam.width + (P.x0 + lp % P.cw);
@@ -1308,8 +1335,9 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
             rng.k0 = (uint32_t)seed;
             rng.k1 = (uint32_t)(seed >> 32);
         }
-        const DScene& S = MULTI ? Sm : P.S;
-        const uint32_t max_depth = MULTI ? md : P.max_depth, flags = MULTI ? fl : P.flags;
+        const DScene& S = MULTI ? P.jobs[job].S : P.S;
+        const uint32_t max_depth = MULTI ? P.jobs[job].max_depth : P.max_depth;
+        const uint32_t flags = MULTI ? P.jobs[job].flags : P.flags;
         NrcHook hook;
         if (NRC) {
             hook.P = &P;
@@ -1345,7 +1373,6 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
         }
         P.radiance[id] = make_float4(ps.L.x, ps.L.y, ps.L.z, MULTI ? L4.w : 0.0f);
         if (NRC) P.aux[id] = hook.aux;
-        (void)job;
     }
     n_ext = warp_sum_u64(n_ext);
     n_sh = warp_sum_u64(n_sh);
@@ -1550,7 +1577,7 @@ static pt_status ensure_restir_buffers(WaveBuffers& w) {
     return PT_OK;
 }
 
-static int g_trace_blocks_per_sm = 0, g_shade_blocks_per_sm = 0, g_shadow_blocks_per_sm = 0, g_tail_blocks_per_sm = 0;
+static int g_trace_blocks_per_sm = 0, g_shadow_blocks_per_sm = 0, g_tail_blocks_per_sm = 0;
 static int g_coop_trace_bps = 0, g_coop_shadow_bps = 0;
 
 // resident blocks per SM of the per-bounce kernels, queried once
@@ -1559,8 +1586,6 @@ static void wf_occupancy() {
     int b = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_trace<false>, 128, 0);
     g_trace_blocks_per_sm = std::max(b, 1);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_shade<false, false>, 128, 0);
-    g_shade_blocks_per_sm = std::max(b, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_shadow<false>, 128, 0);
     g_shadow_blocks_per_sm = std::max(b, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_trace_coop<false>, 128, 0);
@@ -1686,7 +1711,7 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
         key.spp = spp; key.npix_total = npix_total; key.pix_chunk = pix_chunk; key.samp_per_wave = samp_per_wave;
         key.tail_limit = tail_limit; key.tail_grid = tail_grid; key.count = count ? 1u : 0u;
         key.coop = coop ? 1u : 0u;
-        key.sms = sms; key.trace_bps = g_trace_blocks_per_sm; key.shade_bps = g_shade_blocks_per_sm;
+        key.sms = sms; key.trace_bps = g_trace_blocks_per_sm; key.shade_bps = shade_blocks(restir, false);
         key.shadow_bps = g_shadow_blocks_per_sm;
         key.nrc_serial = pt_nrc_serial(o.nrc);
         if (s->wf_graph && s->wf_key.size() == sizeof(key) && std::memcmp(s->wf_key.data(), &key, sizeof(key)) == 0) {
@@ -1785,7 +1810,7 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                         launches += 2;
                     }
                     e = begin(PT_K_SHADE);
-                    const uint32_t shade_grid = sms * g_shade_blocks_per_sm;
+                    const uint32_t shade_grid = sms * shade_blocks(restir, false);
                     if (P.nrc_on) launch_shade<true, false>(s->has_fuzz, shade_grid, st, P, in_q, out_q, k);
                     else if (restir) launch_shade<false, true>(s->has_fuzz, shade_grid, st, P, in_q, out_q, k);
                     else launch_shade<false, false>(s->has_fuzz, shade_grid, st, P, in_q, out_q, k);
@@ -2171,8 +2196,8 @@ static pt_status merged_launches(MergedBatch& m, const WfParams& base, uint32_t 
                 PT_LAUNCH(k_wf_sort_scatter, sms * 2, SORT_THREADS, 0, st, P, in_q);
                 *launches += 2;
             }
-            if (fuzz) PT_LAUNCH((k_wf_shade<false, false, true, true>), sms * g_shade_blocks_per_sm, 128, 0, st, P, in_q, out_q, k);
-            else PT_LAUNCH((k_wf_shade<false, false, false, true>), sms * g_shade_blocks_per_sm, 128, 0, st, P, in_q, out_q, k);
+            if (fuzz) PT_LAUNCH((k_wf_shade<false, false, true, true>), sms * shade_blocks(false, true), 128, 0, st, P, in_q, out_q, k);
+            else PT_LAUNCH((k_wf_shade<false, false, false, true>), sms * shade_blocks(false, true), 128, 0, st, P, in_q, out_q, k);
             PT_LAUNCH((k_wf_shadow<false, true>), sms * g_shadow_blocks_per_sm, 128, 0, st, P);
             *launches += 5;
         }
@@ -2462,7 +2487,7 @@ extern "C" pt_status pt_render_noalloc(pt_scene* s, const pt_camera* camera, uin
                 PT_LAUNCH(k_wf_sort_scatter, sms * 2, SORT_THREADS, 0, st, P, in_q);
                 launches += 2;
             }
-            launch_shade<false, false>(s->has_fuzz, sms * g_shade_blocks_per_sm, st, P, in_q, out_q, k);
+            launch_shade<false, false>(s->has_fuzz, sms * shade_blocks(false, false), st, P, in_q, out_q, k);
             launch_shadow<false>(false, sms, st, P);
             launches += 2;
         }
