@@ -337,12 +337,12 @@ static pt_status launch_megakernel_graph(const std::vector<DJob>& jobs_in, uint3
 }
 
 // ------------------------------------------------------------------ wavefront
-// counters: queue sizes, fetch heads, C_TAIL = 1 once the tail kernel has taken the wave's
+// counters: queue sizes, fetch heads, C_TAIL nonzero once the tail kernel has taken the wave's
 // remaining paths (the per-bounce kernels then have nothing to do), C_FRAME.. the values that
 // change from one call to the next (first sample index, seed: written by k_wf_frame, so the
 // launch sequence of a call is the same every call and can be replayed as a CUDA graph),
 // sort buckets
-enum { C_Q0 = 0, C_Q1 = 1, C_SH = 2, C_HEAD_TRACE = 3, C_HEAD_SHADOW = 4, C_TAIL = 5, C_FRAME = 8,
+enum { C_Q0 = 0, C_Q1 = 1, C_SH = 2, C_HEAD_TRACE = 3, C_HEAD_SHADOW = 4, C_TAIL = 5, C_DONE = 6, C_FRAME = 8,
        C_BUCKETS = 16 };
 constexpr uint32_t MAX_SORT_KEYS = 1024;
 
@@ -456,6 +456,21 @@ __global__ void k_wf_frame(uint32_t* counters, uint32_t first_sample, uint64_t s
     }
 }
 
+// Counters at the start of a wave.  From then on each closest-hit pass leaves them as the
+// passes after it need them (trace_epilogue) and k_wf_shade clears the sort buckets for the
+// next bounce, so no launch is spent on them.
+__device__ __forceinline__ void wave_counters_init(const WfParams& P, uint32_t t, uint32_t n) {
+    if (t == 0) {
+        P.counters[C_Q0] = n;
+        P.counters[C_TAIL] = 0;
+        P.counters[C_SH] = 0;
+        P.counters[C_HEAD_TRACE] = 0;
+        P.counters[C_HEAD_SHADOW] = 0;
+        P.counters[C_DONE] = 0;
+    }
+    for (uint32_t k = t; k < P.n_keys; k += gridDim.x * blockDim.x) P.counters[C_BUCKETS + k] = 0;
+}
+
 // Queue slot t of the first bounce holds path id = t unless the wave is tiled: then within
 // each sample's block of npix slots, slot j holds the pixel of the 8 x 4 tile order (tiles
 // left to right along each group of 4 rows), so that a warp's 32 camera rays cover a compact
@@ -470,11 +485,8 @@ __device__ __forceinline__ uint32_t tiled_path(const WfParams& P, uint32_t t) {
 __global__ void k_wf_raygen(WfParams P) {
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t n = P.npix * P.nsamp;
-    if (t == 0) {
-        P.counters[C_Q0] = n;
-        P.counters[C_TAIL] = 0;
-        atomicAdd(&P.stats[ST_PATHS], (unsigned long long)n);
-    }
+    wave_counters_init(P, t, n);
+    if (t == 0) atomicAdd(&P.stats[ST_PATHS], (unsigned long long)n);
     if (t >= n) return;
     const uint32_t id = P.tiled ? tiled_path(P, t) : t;
     const uint32_t lp = P.pb + id % P.npix;
@@ -595,15 +607,44 @@ __global__ void k_nrc_targets(WfParams P) {
     }
 }
 
-__global__ void k_wf_setup(uint32_t* counters, int out_q, uint32_t n_keys) {
-    const uint32_t t = threadIdx.x;
-    if (t == 0) {
-        counters[out_q] = 0;
-        counters[C_SH] = 0;
-        counters[C_HEAD_TRACE] = 0;
-        counters[C_HEAD_SHADOW] = 0;
+// End of a closest-hit pass: the block's bucket counts go to the global ones, and the last
+// block to arrive turns those into bucket cursors (an exclusive scan) and resets the next
+// queue, the shadow queue and the fetch heads.  As launches of their own (a setup and a scan
+// kernel per bounce) these two cost 4.8 us a bounce.
+__device__ __forceinline__ void trace_epilogue(const WfParams& P, int out_q, const uint32_t* hist) {
+    __shared__ uint32_t last;
+    __syncthreads();
+    for (uint32_t k = threadIdx.x; k < P.n_keys; k += blockDim.x)
+        if (hist[k]) atomicAdd(&P.counters[C_BUCKETS + k], hist[k]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&P.counters[C_DONE], 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!last || threadIdx.x >= 32u) return;
+    __threadfence();
+    const uint32_t lane = threadIdx.x, per = (P.n_keys + 31u) / 32u;
+    const uint32_t b = min(lane * per, P.n_keys), e = min(b + per, P.n_keys);
+    uint32_t sum = 0;
+    for (uint32_t k = b; k < e; ++k) sum += __ldcg(&P.counters[C_BUCKETS + k]);
+    uint32_t x = sum;
+#pragma unroll
+    for (uint32_t off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
     }
-    for (uint32_t k = t; k < n_keys; k += blockDim.x) counters[C_BUCKETS + k] = 0;
+    uint32_t run = x - sum;
+    for (uint32_t k = b; k < e; ++k) {
+        const uint32_t c = __ldcg(&P.counters[C_BUCKETS + k]);
+        P.counters[C_BUCKETS + k] = run;
+        run += c;
+    }
+    if (lane == 0) {
+        P.counters[out_q] = 0;
+        P.counters[C_SH] = 0;
+        P.counters[C_HEAD_TRACE] = 0;
+        P.counters[C_HEAD_SHADOW] = 0;
+        P.counters[C_DONE] = 0;
+    }
 }
 
 __device__ __forceinline__ uint32_t hit_key(const DScene& S, const HitRec& h, uint32_t n_mats) {
@@ -625,14 +666,9 @@ __device__ __forceinline__ uint32_t hit_key(const DScene& S, const HitRec& h, ui
 // blocks per SM (72 / 64 / 56 registers): 3.10 / 2.97 / 3.38 ms; triangles at half / a third /
 // a quarter of the live lanes: 3.20 / 3.12 / 3.15 ms.
 constexpr int TRACE_REFILL = 20, SHADOW_REFILL = 16;
-template <bool COUNT, bool MULTI = false>
-__global__ void __launch_bounds__(128, 8) k_wf_trace(WfParams P, int in_q) {
-    __shared__ uint32_t hist[MAX_SORT_KEYS];
-    if (P.counters[C_TAIL]) return;
+template <bool COUNT, bool MULTI>
+__device__ __forceinline__ void closest_queue(const WfParams& P, int in_q, uint32_t* hist) {
     const bool sort = P.n_keys > 0;
-    if (sort)
-        for (uint32_t k = threadIdx.x; k < P.n_keys; k += blockDim.x) hist[k] = 0;
-    __syncthreads();
     const uint32_t count = P.counters[in_q];
     if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&P.stats[ST_EXT], (unsigned long long)count);
     const uint32_t lane = lane_id(), lt = (1u << lane) - 1u;
@@ -690,34 +726,8 @@ __global__ void __launch_bounds__(128, 8) k_wf_trace(WfParams P, int in_q) {
             continue;
         }
         bool fail = false;
-        if (2 * __popc(mt) >= __popc(mn)) {
-            if (r.tri_mask != 0u) {
-                const uint32_t ti = r.tri_base + (uint32_t)(__ffs(r.tri_mask) - 1);
-                r.tri_mask &= r.tri_mask - 1u;
-                const float4 a = __ldg(tris + 3u * ti), b = __ldg(tris + 3u * ti + 1), c = __ldg(tris + 3u * ti + 2);
-                float t, u, w;
-                if (tri_hit(r.wr, xyz(a), xyz(b), xyz(c), __int_as_float(0x7f800000), t, u, w)) {
-                    const uint32_t orig = __float_as_uint(a.w);
-                    if (t < h.t || (t == h.t && orig < best_orig)) {
-                        h.t = t; h.tri = ti; best_orig = orig; best_code = __float_as_uint(b.w);
-                    }
-                }
-            }
-        } else if (alive && r.tri_mask == 0u) {
-            // more visits than nodes mean a malformed tree
-            if (r.budget-- <= 1u) {
-                const uint32_t nn = MULTI ? (uint32_t)P.jobs[job].S.n_nodes : (uint32_t)P.S.n_nodes;
-                if (nn != 0u) atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 4u);
-                h.tri = PT_NO_HIT;
-                fail = true;
-            } else {
-                lane_closest_node<COUNT>(nodes, r, h.t, stack, tc);
-                if (r.sp > PT_STACK) { atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 1u); fail = true; }
-            }
-        }
-        __syncwarp();
-        if (alive && (r.tri_mask == 0u || fail)) {
-            // the next child whose entry distance is still within the closest hit
+        // the next child whose entry distance is still within the closest hit, or the end
+        auto advance = [&]() {
             bool done = fail;
             while (!done && !(r.near_t <= h.t)) {
                 if (r.sp == 0) { done = true; break; }
@@ -730,8 +740,43 @@ __global__ void __launch_bounds__(128, 8) k_wf_trace(WfParams P, int in_q) {
                 pend = true;
                 r.tri_mask = 0u;
             }
+        };
+        if (2 * __popc(mt) >= __popc(mn)) {
+            if (r.tri_mask != 0u) {
+                const uint32_t ti = r.tri_base + (uint32_t)(__ffs(r.tri_mask) - 1);
+                r.tri_mask &= r.tri_mask - 1u;
+                const float4 a = __ldg(tris + 3u * ti), b = __ldg(tris + 3u * ti + 1), c = __ldg(tris + 3u * ti + 2);
+                float t, u, w;
+                if (tri_hit(r.wr, xyz(a), xyz(b), xyz(c), __int_as_float(0x7f800000), t, u, w)) {
+                    const uint32_t orig = __float_as_uint(a.w);
+                    if (t < h.t || (t == h.t && orig < best_orig)) {
+                        h.t = t; h.tri = ti; best_orig = orig; best_code = __float_as_uint(b.w);
+                    }
+                }
+                if (r.tri_mask == 0u) advance();
+            }
+            __syncwarp();
+        } else {
+            // nodes until a third of the lanes that were live have come to a leaf or to their end
+            const int stay = 2 * __popc(mt | mn) / 3;
+            uint32_t go;
+            do {
+                if (alive && r.tri_mask == 0u) {
+                    // more visits than nodes mean a malformed tree
+                    if (r.budget-- <= 1u) {
+                        const uint32_t nn = MULTI ? (uint32_t)P.jobs[job].S.n_nodes : (uint32_t)P.S.n_nodes;
+                        if (nn != 0u) atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 4u);
+                        h.tri = PT_NO_HIT;
+                        fail = true;
+                    } else {
+                        lane_closest_node<COUNT>(nodes, r, h.t, stack, tc);
+                        if (r.sp > PT_STACK) { atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 1u); fail = true; }
+                    }
+                    if (r.tri_mask == 0u || fail) advance();
+                }
+                go = __ballot_sync(0xffffffffu, alive && r.tri_mask == 0u);
+            } while (__popc(go) > stay);
         }
-        __syncwarp();
     }
     if (COUNT) {
         const unsigned long long nn = warp_sum_u64(tc.nodes), nt = warp_sum_u64(tc.tris),
@@ -742,28 +787,139 @@ __global__ void __launch_bounds__(128, 8) k_wf_trace(WfParams P, int in_q) {
             atomicAdd(&P.stats[ST_TRIS], nt);
         }
     }
-    if (sort) {
-        __syncthreads();
-        for (uint32_t k = threadIdx.x; k < P.n_keys; k += blockDim.x)
-            if (hist[k]) atomicAdd(&P.counters[C_BUCKETS + k], hist[k]);
+}
+
+// Persistent shadow any-hit over the shadow queue, in the same stages; an unoccluded shadow
+// ray adds its contribution to its path's radiance, at the refill too: the three dependent
+// accesses of that addition would otherwise stall the warp for one or two lanes at a time
+// (1080p CAD frame, 8.3M paths: 1.75 ms one ray per lane to the end, 1.37 ms in stages, 1.27
+// with the additions at the refill).
+template <bool COUNT, bool MULTI>
+__device__ __forceinline__ void shadow_queue(const WfParams& P) {
+    const uint32_t count = P.counters[C_SH];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && count) atomicAdd(&P.stats[ST_SHADOW], (unsigned long long)count);
+    const uint32_t lane = lane_id(), lt = (1u << lane) - 1u;
+    TravCount tc = {0, 0, 0};
+    LaneRay r;
+    uint32_t stack[PT_STACK + PT_STACK_SLACK];
+    uint32_t slot = 0, id = 0, job = 0;
+    float tmax = 0.0f;
+    const uint4* nodes = P.S.nodes;
+    const float4* tris = P.S.tris;
+    bool alive = false, pend = false, drained = count == 0u;
+    r.tri_mask = 0u;
+    for (;;) {
+        const uint32_t mt = __ballot_sync(0xffffffffu, r.tri_mask != 0u);
+        const uint32_t mn = __ballot_sync(0xffffffffu, alive && r.tri_mask == 0u);
+        const uint32_t idle = ~(mt | mn);
+        if (__popc(idle) >= (drained ? 32 : SHADOW_REFILL)) {
+            if (pend) {
+                const float4 c = P.sh_c[slot];
+                float4 L = P.radiance[id];
+                L.x += c.x; L.y += c.y; L.z += c.z;
+                P.radiance[id] = L;
+                pend = false;
+            }
+            if (drained) break;
+            const uint32_t want = __popc(idle);
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(&P.counters[C_HEAD_SHADOW], want);
+            base = __shfl_sync(0xffffffffu, base, 0);
+            drained = base + want >= count;
+            const uint32_t mine = base + __popc(idle & lt);
+            if (!alive && mine < count) {
+                slot = mine;
+                const float4 so = P.sh_o[slot], sd = P.sh_d[slot];
+                uint32_t nn;
+                if (MULTI) {
+                    // merged batch waves: the job rides in the w word of the contribution
+                    job = __float_as_uint(P.sh_c[slot].w);
+                    nodes = P.jobs[job].S.nodes;
+                    tris = P.jobs[job].S.tris;
+                    nn = (uint32_t)P.jobs[job].S.n_nodes;
+                } else {
+                    nn = (uint32_t)P.S.n_nodes;
+                }
+                tmax = so.w;
+                id = __float_as_uint(sd.w);
+                lane_ray_init(xyz(so), xyz(sd), nn, r);
+                alive = true;
+            }
+            continue;
+        }
+        auto finish = [&](bool occluded) {
+            alive = false;
+            pend = !occluded;
+            r.tri_mask = 0u;
+        };
+        auto advance = [&]() {
+            if (r.node != PT_NO_HIT) return;
+            if (r.sp == 0) finish(false);
+            else r.node = stack[--r.sp];
+        };
+        if (2 * __popc(mt) >= __popc(mn)) {
+            if (r.tri_mask != 0u) {
+                const uint32_t ti = r.tri_base + (uint32_t)(__ffs(r.tri_mask) - 1);
+                r.tri_mask &= r.tri_mask - 1u;
+                if (COUNT) tc.tris++;
+                const float4 a = __ldg(tris + 3u * ti), b = __ldg(tris + 3u * ti + 1), c = __ldg(tris + 3u * ti + 2);
+                float t, u, w;
+                if (tri_hit(r.wr, xyz(a), xyz(b), xyz(c), tmax, t, u, w)) finish(true);
+                else if (r.tri_mask == 0u) advance();
+            }
+            __syncwarp();
+        } else {
+            const int stay = 2 * __popc(mt | mn) / 3;
+            uint32_t go;
+            do {
+                if (alive && r.tri_mask == 0u) {
+                    if (r.budget-- <= 1u) {
+                        const uint32_t nn = MULTI ? (uint32_t)P.jobs[job].S.n_nodes : (uint32_t)P.S.n_nodes;
+                        if (nn != 0u) atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 4u);
+                        finish(false);
+                    } else {
+                        lane_any_node<COUNT>(nodes, r, tmax, stack, tc);
+                        if (r.sp > PT_STACK) {
+                            atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 1u);
+                            finish(true);
+                        } else if (r.tri_mask == 0u) {
+                            advance();
+                        }
+                    }
+                }
+                go = __ballot_sync(0xffffffffu, alive && r.tri_mask == 0u);
+            } while (__popc(go) > stay);
+        }
+    }
+    if (COUNT) {
+        const unsigned long long nn = warp_sum_u64(tc.nodes), nt = warp_sum_u64(tc.tris),
+                                 nb = warp_sum_u64(tc.boxes);
+        if (lane == 0) {
+            atomicAdd(&P.stats[ST_SH_BOXES], nb);
+            atomicAdd(&P.stats[ST_SH_NODES], nn);
+            atomicAdd(&P.stats[ST_SH_TRIS], nt);
+        }
     }
 }
 
-// exclusive scan of the bucket counts into bucket cursors (one block)
-__global__ void k_wf_sort_scan(uint32_t* counters, uint32_t n_keys) {
-    if (counters[C_TAIL]) return;
-    __shared__ uint32_t part[MAX_SORT_KEYS];
-    const uint32_t t = threadIdx.x;
-    const uint32_t v = t < n_keys ? counters[C_BUCKETS + t] : 0u;
-    part[t] = v;
-    __syncthreads();
-    for (uint32_t off = 1; off < blockDim.x; off <<= 1) {
-        const uint32_t a = t >= off ? part[t - off] : 0u;
+// The rays of a bounce: its closest-hit queue, then the shadow queue of the bounce before.  The
+// two don't depend on each other, and in one launch the warps that find the first queue empty
+// go on with the second while the longest rays of the first are finished (a launch each left
+// the chip to those rays twice a bounce).  what: RAYS_CLOSEST | RAYS_SHADOW; timed calls
+// launch them one by one.
+enum { RAYS_CLOSEST = 1, RAYS_SHADOW = 2 };
+
+template <bool COUNT, bool MULTI = false>
+__global__ void __launch_bounds__(128, 8) k_wf_rays(WfParams P, int in_q, int out_q, int what) {
+    __shared__ uint32_t hist[MAX_SORT_KEYS];
+    if (P.counters[C_TAIL]) return;
+    if (what & RAYS_CLOSEST) {
+        for (uint32_t k = threadIdx.x; k < P.n_keys; k += blockDim.x) hist[k] = 0;
         __syncthreads();
-        part[t] += a;
-        __syncthreads();
+        closest_queue<COUNT, MULTI>(P, in_q, hist);
     }
-    if (t < n_keys) counters[C_BUCKETS + t] = part[t] - v;
+    if (what & RAYS_SHADOW) shadow_queue<COUNT, MULTI>(P);
+    if (what & RAYS_CLOSEST) trace_epilogue(P, out_q, hist);
 }
 
 // Counting-sort scatter: each block ranks a chunk of SORT_ITEMS x SORT_THREADS slots in shared
@@ -955,6 +1111,9 @@ constexpr int shade_blocks(bool ris, bool multi) { return ris || multi ? 4 : 5; 
 template <bool NRC, bool RIS, bool FUZZ = true, bool MULTI = false>
 __global__ void __launch_bounds__(128, shade_blocks(RIS, MULTI)) k_wf_shade(WfParams P, int in_q, int out_q, uint32_t k) {
     if (P.counters[C_TAIL]) return;
+    // the scatter pass is done with its cursors: zero counts for the next closest-hit pass
+    if (blockIdx.x == 0)
+        for (uint32_t b = threadIdx.x; b < P.n_keys; b += blockDim.x) P.counters[C_BUCKETS + b] = 0;
     const uint32_t count = P.counters[in_q];
     const uint32_t sbase = wf_sample_base(P);
     const uint64_t seed = wf_seed(P);
@@ -1067,107 +1226,6 @@ __global__ void __launch_bounds__(128, shade_blocks(RIS, MULTI)) k_wf_shade(WfPa
     if (lane == 0 && rr_cnt) atomicAdd(&P.stats[ST_RR], rr_cnt);
 }
 
-// Persistent shadow any-hit over the shadow queue, in the same stages; an unoccluded shadow
-// ray adds its contribution to its path's radiance, at the refill too: the three dependent
-// accesses of that addition would otherwise stall the warp for one or two lanes at a time
-// (1080p CAD frame, 8.3M paths: 1.75 ms one ray per lane to the end, 1.37 ms in stages, 1.27
-// with the additions at the refill).
-template <bool COUNT, bool MULTI = false>
-__global__ void __launch_bounds__(128, 8) k_wf_shadow(WfParams P) {
-    const uint32_t count = P.counters[C_SH];
-    if (blockIdx.x == 0 && threadIdx.x == 0 && count) atomicAdd(&P.stats[ST_SHADOW], (unsigned long long)count);
-    const uint32_t lane = lane_id(), lt = (1u << lane) - 1u;
-    TravCount tc = {0, 0, 0};
-    LaneRay r;
-    uint32_t stack[PT_STACK + PT_STACK_SLACK];
-    uint32_t slot = 0, id = 0, job = 0;
-    float tmax = 0.0f;
-    const uint4* nodes = P.S.nodes;
-    const float4* tris = P.S.tris;
-    bool alive = false, pend = false, drained = count == 0u;
-    r.tri_mask = 0u;
-    for (;;) {
-        const uint32_t mt = __ballot_sync(0xffffffffu, r.tri_mask != 0u);
-        const uint32_t mn = __ballot_sync(0xffffffffu, alive && r.tri_mask == 0u);
-        const uint32_t idle = ~(mt | mn);
-        if (__popc(idle) >= (drained ? 32 : SHADOW_REFILL)) {
-            if (pend) {
-                const float4 c = P.sh_c[slot];
-                float4 L = P.radiance[id];
-                L.x += c.x; L.y += c.y; L.z += c.z;
-                P.radiance[id] = L;
-                pend = false;
-            }
-            if (drained) break;
-            const uint32_t want = __popc(idle);
-            uint32_t base = 0;
-            if (lane == 0) base = atomicAdd(&P.counters[C_HEAD_SHADOW], want);
-            base = __shfl_sync(0xffffffffu, base, 0);
-            drained = base + want >= count;
-            const uint32_t mine = base + __popc(idle & lt);
-            if (!alive && mine < count) {
-                slot = mine;
-                const float4 so = P.sh_o[slot], sd = P.sh_d[slot];
-                uint32_t nn;
-                if (MULTI) {
-                    // merged batch waves: the job rides in the w word of the contribution
-                    job = __float_as_uint(P.sh_c[slot].w);
-                    nodes = P.jobs[job].S.nodes;
-                    tris = P.jobs[job].S.tris;
-                    nn = (uint32_t)P.jobs[job].S.n_nodes;
-                } else {
-                    nn = (uint32_t)P.S.n_nodes;
-                }
-                tmax = so.w;
-                id = __float_as_uint(sd.w);
-                lane_ray_init(xyz(so), xyz(sd), nn, r);
-                alive = true;
-            }
-            continue;
-        }
-        bool done = false, occ = false;
-        if (2 * __popc(mt) >= __popc(mn)) {
-            if (r.tri_mask != 0u) {
-                const uint32_t ti = r.tri_base + (uint32_t)(__ffs(r.tri_mask) - 1);
-                r.tri_mask &= r.tri_mask - 1u;
-                if (COUNT) tc.tris++;
-                const float4 a = __ldg(tris + 3u * ti), b = __ldg(tris + 3u * ti + 1), c = __ldg(tris + 3u * ti + 2);
-                float t, u, w;
-                if (tri_hit(r.wr, xyz(a), xyz(b), xyz(c), tmax, t, u, w)) occ = done = true;
-            }
-        } else if (alive && r.tri_mask == 0u) {
-            if (r.budget-- <= 1u) {
-                const uint32_t nn = MULTI ? (uint32_t)P.jobs[job].S.n_nodes : (uint32_t)P.S.n_nodes;
-                if (nn != 0u) atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 4u);
-                done = true;
-            } else {
-                lane_any_node<COUNT>(nodes, r, tmax, stack, tc);
-                if (r.sp > PT_STACK) { atomicOr(MULTI ? P.jobs[job].S.err : P.S.err, 1u); occ = done = true; }
-            }
-        }
-        __syncwarp();
-        if (alive && !done && r.tri_mask == 0u && r.node == PT_NO_HIT) {
-            if (r.sp == 0) done = true;
-            else r.node = stack[--r.sp];
-        }
-        if (done) {
-            alive = false;
-            pend = !occ;
-            r.tri_mask = 0u;
-        }
-        __syncwarp();
-    }
-    if (COUNT) {
-        const unsigned long long nn = warp_sum_u64(tc.nodes), nt = warp_sum_u64(tc.tris),
-                                 nb = warp_sum_u64(tc.boxes);
-        if (lane == 0) {
-            atomicAdd(&P.stats[ST_SH_BOXES], nb);
-            atomicAdd(&P.stats[ST_SH_NODES], nn);
-            atomicAdd(&P.stats[ST_SH_TRIS], nt);
-        }
-    }
-}
-
 // Cooperative variants of the two traversal passes (PT_TRAVERSAL_COOP): a group of COOP_W = 8
 // lanes carries one ray (pt_device.cuh, coop_*), so a warp holds 4 rays and its lanes test a
 // node's 8 child boxes, or a node's leaf triangles, side by side.  A warp claims 32 queue
@@ -1199,7 +1257,7 @@ __device__ __forceinline__ void coop_hand_out(uint32_t* head, uint32_t count, ui
 }
 
 template <bool COUNT>
-__global__ void __launch_bounds__(128) k_wf_trace_coop(WfParams P, int in_q) {
+__global__ void __launch_bounds__(128) k_wf_trace_coop(WfParams P, int in_q, int out_q) {
     __shared__ uint32_t hist[MAX_SORT_KEYS];
     __shared__ CoopShared gsh[128 / COOP_W];
     if (P.counters[C_TAIL]) return;
@@ -1248,15 +1306,12 @@ __global__ void __launch_bounds__(128) k_wf_trace_coop(WfParams P, int in_q) {
             atomicAdd(&P.stats[ST_TRIS], nt);
         }
     }
-    if (sort) {
-        __syncthreads();
-        for (uint32_t k = threadIdx.x; k < P.n_keys; k += blockDim.x)
-            if (hist[k]) atomicAdd(&P.counters[C_BUCKETS + k], hist[k]);
-    }
+    trace_epilogue(P, out_q, hist);
 }
 
 template <bool COUNT>
 __global__ void __launch_bounds__(128) k_wf_shadow_coop(WfParams P) {
+    if (P.counters[C_TAIL]) return;
     __shared__ CoopShared gsh[128 / COOP_W];
     const uint32_t count = P.counters[C_SH];
     if (blockIdx.x == 0 && threadIdx.x == 0 && count) atomicAdd(&P.stats[ST_SHADOW], (unsigned long long)count);
@@ -1301,16 +1356,20 @@ __global__ void __launch_bounds__(128) k_wf_shadow_coop(WfParams P) {
 
 // Tail of a wave: when few paths are left, a per-bounce kernel lasts about as long as its
 // slowest ray (a chain of dependent node and triangle loads), and the wave pays that once per
-// stage and bounce.  This kernel takes the remaining queue instead and carries each path to
-// its end in one thread: closest hit, shade_vertex_h (the same per-vertex code and random
+// stage and bounce.  This kernel takes the remaining queue instead, its rays just traced, and
+// carries each path to its end in one thread: closest hit, shade_vertex_h (the same per-vertex code and random
 // numbers as k_wf_shade), then the shadow ray, whose contribution is added after the vertex's
 // own terms exactly as k_wf_shadow adds it.  It appends nothing, so the later per-bounce
 // launches of the wave find empty queues (and C_TAIL makes the rest of this bounce skip).
 template <bool NRC, bool COUNT, bool RIS, bool FUZZ = true, bool MULTI = false>
 __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32_t k0, uint32_t limit) {
+    // C_TAIL holds the bounce (plus one) at which the tail took the wave: a launch for a later
+    // bounce finds a queue that no pass has written
+    const uint32_t taken = P.counters[C_TAIL];
+    if (taken != 0u && taken != k0 + 1u) return;
     const uint32_t count = P.counters[in_q];
     if (count == 0 || count > limit) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) P.counters[C_TAIL] = 1u;
+    if (blockIdx.x == 0 && threadIdx.x == 0) P.counters[C_TAIL] = k0 + 1u;
     const uint32_t sbase = wf_sample_base(P);
     const uint64_t seed = wf_seed(P);
     unsigned long long n_ext = 0, n_sh = 0, n_rr = 0;
@@ -1345,11 +1404,16 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
             hook.aux = P.aux[id];
         }
         float3 o = xyz(ro), d = xyz(rd);
+        const float4 hh = P.hit[i];      // of this bounce's rays, already traced
         for (uint32_t k = k0;; ++k) {
             HitRec h;
-            if (COUNT) trace_closest_t<true, true>(S, o, d, __int_as_float(0x7f800000), h, tc);
-            else trace_closest(S, o, d, __int_as_float(0x7f800000), h);
-            n_ext++;
+            if (k == k0) {
+                h.t = hh.x; h.u = h.v = 0.0f; h.tri = __float_as_uint(hh.w);
+            } else {
+                if (COUNT) trace_closest_t<true, true>(S, o, d, __int_as_float(0x7f800000), h, tc);
+                else trace_closest(S, o, d, __int_as_float(0x7f800000), h);
+                n_ext++;
+            }
             rng.k = k;
             ShadeOut so;
             int r;
@@ -1400,10 +1464,7 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
 // ---- merged batch waves: raygen and accumulation over a wave's segments
 __global__ void k_wfm_raygen(WfParams P, uint32_t n_paths) {
     const uint32_t id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id == 0) {
-        P.counters[C_Q0] = n_paths;
-        P.counters[C_TAIL] = 0;
-    }
+    wave_counters_init(P, id, n_paths);
     if (id >= n_paths) return;
     const uint32_t si = wfm_seg_of(P, id);
     const WfmSeg g = P.segs[si];
@@ -1577,33 +1638,31 @@ static pt_status ensure_restir_buffers(WaveBuffers& w) {
     return PT_OK;
 }
 
-static int g_trace_blocks_per_sm = 0, g_shadow_blocks_per_sm = 0, g_tail_blocks_per_sm = 0;
+static int g_rays_blocks_per_sm = 0, g_tail_blocks_per_sm = 0;
 static int g_coop_trace_bps = 0, g_coop_shadow_bps = 0;
 
 // resident blocks per SM of the per-bounce kernels, queried once
 static void wf_occupancy() {
-    if (g_trace_blocks_per_sm != 0) return;
+    if (g_rays_blocks_per_sm != 0) return;
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_trace<false>, 128, 0);
-    g_trace_blocks_per_sm = std::max(b, 1);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_shadow<false>, 128, 0);
-    g_shadow_blocks_per_sm = std::max(b, 1);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_rays<false>, 128, 0);
+    g_rays_blocks_per_sm = std::max(b, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_trace_coop<false>, 128, 0);
     g_coop_trace_bps = std::max(b, 1);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_wf_shadow_coop<false>, 128, 0);
     g_coop_shadow_bps = std::max(b, 1);
 }
 
-// the closest-hit and shadow passes, per-lane or cooperative (the same hits and counts)
-template <bool COUNT>
-static void launch_trace(bool coop, int sms, cudaStream_t st, const WfParams& P, int in_q) {
-    if (coop) PT_LAUNCH(k_wf_trace_coop<COUNT>, sms * g_coop_trace_bps, 128, 0, st, P, in_q);
-    else PT_LAUNCH(k_wf_trace<COUNT>, sms * g_trace_blocks_per_sm, 128, 0, st, P, in_q);
+// the rays of a bounce (k_wf_rays)
+template <bool COUNT, bool MULTI = false>
+static void launch_rays(int sms, cudaStream_t st, const WfParams& P, int in_q, int out_q, int what) {
+    PT_LAUNCH((k_wf_rays<COUNT, MULTI>), sms * g_rays_blocks_per_sm, 128, 0, st, P, in_q, out_q, what);
 }
+// the same passes with one ray per 8 lanes (the same hits and counts)
 template <bool COUNT>
-static void launch_shadow(bool coop, int sms, cudaStream_t st, const WfParams& P) {
-    if (coop) PT_LAUNCH(k_wf_shadow_coop<COUNT>, sms * g_coop_shadow_bps, 128, 0, st, P);
-    else PT_LAUNCH(k_wf_shadow<COUNT>, sms * g_shadow_blocks_per_sm, 128, 0, st, P);
+static void launch_rays_coop(int sms, cudaStream_t st, const WfParams& P, int in_q, int out_q, int what) {
+    if (what & RAYS_CLOSEST) PT_LAUNCH(k_wf_trace_coop<COUNT>, sms * g_coop_trace_bps, 128, 0, st, P, in_q, out_q);
+    if (what & RAYS_SHADOW) PT_LAUNCH(k_wf_shadow_coop<COUNT>, sms * g_coop_shadow_bps, 128, 0, st, P);
 }
 
 pt_status pt_wavefront_tail_limit(int* out) {
@@ -1621,7 +1680,7 @@ pt_status pt_wavefront_tail_limit(int* out) {
 struct WfGraphKey {
     WfParams P;             // with the per-wave fields cleared
     uint32_t spp, npix_total, pix_chunk, samp_per_wave, tail_limit, tail_grid, count, coop;
-    int sms, trace_bps, shade_bps, shadow_bps;
+    int sms, rays_bps, shade_bps;
     uint64_t nrc_serial;    // the radiance cache the launches read and train (0: none)
 };
 
@@ -1629,21 +1688,34 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                                   pt_accum* acc, const pt_render_opts& o, cudaStream_t user_st) {
     cudaStream_t st = user_st;   // the stream the wave loops below issue to (a capture stream while capturing)
     const uint32_t npix_total = acc->width * acc->height;
-    uint32_t cap = o.wave_paths ? o.wave_paths : (1u << 21);
-    cap = std::max(cap, 32u);
+    // automatic wave: 2^23 paths (1.4 GB of queues), or 2^21 where there is no room for that and
+    // in frames that train the cache (a wave is a training set).  Every pass of a wave ends with
+    // the chip waiting for its longest rays, so few large waves beat many small ones: 2^21 /
+    // 2^22 / 2^23 / 2^24 paths a wave, 512 x 512 still of 25 samples 10.12 / 7.93 / 6.84 / 6.84
+    // ms, glass scene at 1917 x 1079 and 2 samples 5.85 / 4.20 / 4.21 / 4.23.
+    constexpr uint32_t LARGE_WAVE = 1u << 23, SMALL_WAVE = 1u << 21;
+    const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train);
+    uint32_t cap = std::max(o.wave_paths ? o.wave_paths : large ? LARGE_WAVE : SMALL_WAVE, 32u);
     // waves hold whole samples of a pixel range: pixel chunk <= cap, then samples per wave;
     // with ReSTIR the chunk is the whole window (the spatial pass reads any pixel of it)
     const bool restir = o.restir != nullptr;
     const bool coop = o.traversal == PT_TRAVERSAL_COOP;
-    const uint32_t pix_chunk = restir ? npix_total : std::min(npix_total, cap);
-    const uint32_t samp_per_wave = std::max(1u, std::min(spp, cap / pix_chunk));
-    pt_status r = ensure_wave(s->wave, pix_chunk * samp_per_wave);
-    if (r != PT_OK) return r;
     WaveBuffers& w = s->wave;
-    if (restir) {
-        r = ensure_restir_buffers(w);
-        if (r != PT_OK) return r;
+    uint32_t pix_chunk = 0, samp_per_wave = 0;
+    auto buffers = [&]() -> pt_status {
+        pix_chunk = restir ? npix_total : std::min(npix_total, cap);
+        samp_per_wave = std::max(1u, std::min(spp, cap / pix_chunk));
+        const pt_status e = ensure_wave(w, pix_chunk * samp_per_wave);
+        return e == PT_OK && restir ? ensure_restir_buffers(w) : e;
+    };
+    pt_status r = buffers();
+    if (r == PT_ERR_OOM && large) {
+        cudaGetLastError();
+        pt_free_wave(w);
+        cap = SMALL_WAVE;
+        r = buffers();
     }
+    if (r != PT_OK) return r;
     const bool sort = o.sort_by_material == 1 || (o.sort_by_material < 0 && s->n_mats + 2 <= MAX_SORT_KEYS && s->n_mats > 1);
     const uint32_t n_keys = (sort && s->n_mats + 2 <= MAX_SORT_KEYS) ? s->n_mats + 2 : 0;
     wf_occupancy();
@@ -1711,8 +1783,7 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
         key.spp = spp; key.npix_total = npix_total; key.pix_chunk = pix_chunk; key.samp_per_wave = samp_per_wave;
         key.tail_limit = tail_limit; key.tail_grid = tail_grid; key.count = count ? 1u : 0u;
         key.coop = coop ? 1u : 0u;
-        key.sms = sms; key.trace_bps = g_trace_blocks_per_sm; key.shade_bps = shade_blocks(restir, false);
-        key.shadow_bps = g_shadow_blocks_per_sm;
+        key.sms = sms; key.rays_bps = g_rays_blocks_per_sm; key.shade_bps = shade_blocks(restir, false);
         key.nrc_serial = pt_nrc_serial(o.nrc);
         if (s->wf_graph && s->wf_key.size() == sizeof(key) && std::memcmp(s->wf_key.data(), &key, sizeof(key)) == 0) {
             PT_CUDA_TRY(cudaGraphLaunch(s->wf_graph, user_st));
@@ -1766,10 +1837,24 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                 PT_LAUNCH(k_wf_raygen, (n + 255) / 256, 256, 0, st, P);
                 end(e);
                 ++launches;
+                // shadow rays of one bounce and closest hits of the next share a launch, except in
+                // timed calls and cooperative traversal; at max_depth no vertex sends a shadow ray
+                const bool split = timed || coop;
+                auto rays = [&](int in_q, int out_q, int what) {
+                    if (coop) {
+                        if (count) launch_rays_coop<true>(sms, st, P, in_q, out_q, what);
+                        else launch_rays_coop<false>(sms, st, P, in_q, out_q, what);
+                    } else {
+                        if (count) launch_rays<true>(sms, st, P, in_q, out_q, what);
+                        else launch_rays<false>(sms, st, P, in_q, out_q, what);
+                    }
+                    ++launches;
+                };
                 for (uint32_t k = 0; k <= max_depth; ++k) {
                     const int in_q = (int)(k & 1u), out_q = (int)((k + 1) & 1u);
-                    PT_LAUNCH(k_wf_setup, 1, 256, 0, st, w.counters, out_q, n_keys);
-                    ++launches;
+                    e = begin(PT_K_TRACE);
+                    rays(in_q, out_q, split || k == 0 ? RAYS_CLOSEST : RAYS_CLOSEST | RAYS_SHADOW);
+                    end(e);
                     if (tail_limit && !(restir && k == 0)) {
                         // at the forced bounce the tail kernel takes the paths whatever their number
                         const bool force = P.tail_bounce != 0 && k == P.tail_bounce;
@@ -1790,17 +1875,11 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                         ++launches;
                         if (force) break;   // no path is left for the later bounces
                     }
-                    e = begin(PT_K_TRACE);
-                    if (count) launch_trace<true>(coop, sms, st, P, in_q);
-                    else launch_trace<false>(coop, sms, st, P, in_q);
-                    end(e);
-                    ++launches;
                     if (n_keys) {
                         e = begin(PT_K_SORT);
-                        PT_LAUNCH(k_wf_sort_scan, 1, MAX_SORT_KEYS, 0, st, w.counters, n_keys);
                         PT_LAUNCH(k_wf_sort_scatter, sms * 2, SORT_THREADS, 0, st, P, in_q);
                         end(e);
-                        launches += 2;
+                        ++launches;
                     }
                     if (restir && k == 0) {
                         e = begin(PT_K_RESTIR);
@@ -1815,11 +1894,12 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                     else if (restir) launch_shade<false, true>(s->has_fuzz, shade_grid, st, P, in_q, out_q, k);
                     else launch_shade<false, false>(s->has_fuzz, shade_grid, st, P, in_q, out_q, k);
                     end(e);
-                    e = begin(PT_K_SHADOW);
-                    if (count) launch_shadow<true>(coop, sms, st, P);
-                    else launch_shadow<false>(coop, sms, st, P);
-                    end(e);
-                    launches += 2;
+                    ++launches;
+                    if (split && k < max_depth) {
+                        e = begin(PT_K_SHADOW);
+                        rays(in_q, out_q, RAYS_SHADOW);
+                        end(e);
+                    }
                 }
                 if (P.nrc_on) {
                     // cache inference for the paths that ended at their second diffuse-ish vertex,
@@ -2187,19 +2267,16 @@ static pt_status merged_launches(MergedBatch& m, const WfParams& base, uint32_t 
         ++*launches;
         for (uint32_t k = 0; k <= max_depth; ++k) {
             const int in_q = (int)(k & 1u), out_q = (int)((k + 1) & 1u);
-            PT_LAUNCH(k_wf_setup, 1, 256, 0, st, m.wave.counters, out_q, P.n_keys);
+            launch_rays<false, true>(sms, st, P, in_q, out_q, k ? RAYS_CLOSEST | RAYS_SHADOW : RAYS_CLOSEST);
             if (fuzz) PT_LAUNCH((k_wf_tail<false, false, false, true, true>), tail_grid, 128, 0, st, P, in_q, k, tail_limit);
             else PT_LAUNCH((k_wf_tail<false, false, false, false, true>), tail_grid, 128, 0, st, P, in_q, k, tail_limit);
-            PT_LAUNCH((k_wf_trace<false, true>), sms * g_trace_blocks_per_sm, 128, 0, st, P, in_q);
             if (P.n_keys) {
-                PT_LAUNCH(k_wf_sort_scan, 1, MAX_SORT_KEYS, 0, st, m.wave.counters, P.n_keys);
                 PT_LAUNCH(k_wf_sort_scatter, sms * 2, SORT_THREADS, 0, st, P, in_q);
-                *launches += 2;
+                ++*launches;
             }
             if (fuzz) PT_LAUNCH((k_wf_shade<false, false, true, true>), sms * shade_blocks(false, true), 128, 0, st, P, in_q, out_q, k);
             else PT_LAUNCH((k_wf_shade<false, false, false, true>), sms * shade_blocks(false, true), 128, 0, st, P, in_q, out_q, k);
-            PT_LAUNCH((k_wf_shadow<false, true>), sms * g_shadow_blocks_per_sm, 128, 0, st, P);
-            *launches += 5;
+            *launches += 3;
         }
         PT_LAUNCH(k_wfm_accum, (m.wave_pix[w] + 255) / 256, 256, 0, st, P, m.wave_pix[w]);
         ++*launches;
@@ -2377,7 +2454,7 @@ extern "C" pt_status pt_render_batch(const pt_job* jobs, uint32_t n_jobs, const 
 // pt_render_noalloc serves them: the same wavefront kernels as pt_render, but the work
 // queues live in the fixed-size array below, which every GPU that loads this library keeps
 // until the process exits.  The kernels themselves reset every counter that must start at
-// zero (raygen sets the input queue size, the per-bounce setup kernel clears the output
+// zero (raygen sets the input queue size, the closest-hit and shade passes clear the next
 // queue, the shadow queue, the fetch heads and the sort buckets) and initialise every path
 // slot they read, so stale contents from an earlier call are never used.
 constexpr uint32_t NOALLOC_MAX_PATHS = 16384;
@@ -2479,17 +2556,14 @@ extern "C" pt_status pt_render_noalloc(pt_scene* s, const pt_camera* camera, uin
         ++launches;
         for (uint32_t k = 0; k <= max_depth; ++k) {
             const int in_q = (int)(k & 1u), out_q = (int)((k + 1) & 1u);
-            PT_LAUNCH(k_wf_setup, 1, 256, 0, st, w.counters, out_q, n_keys);
-            launch_trace<false>(false, sms, st, P, in_q);
-            launches += 2;
+            launch_rays<false>(sms, st, P, in_q, out_q, k ? RAYS_CLOSEST | RAYS_SHADOW : RAYS_CLOSEST);
+            ++launches;
             if (n_keys) {
-                PT_LAUNCH(k_wf_sort_scan, 1, MAX_SORT_KEYS, 0, st, w.counters, n_keys);
                 PT_LAUNCH(k_wf_sort_scatter, sms * 2, SORT_THREADS, 0, st, P, in_q);
-                launches += 2;
+                ++launches;
             }
             launch_shade<false, false>(s->has_fuzz, sms * shade_blocks(false, false), st, P, in_q, out_q, k);
-            launch_shadow<false>(false, sms, st, P);
-            launches += 2;
+            ++launches;
         }
         PT_LAUNCH(k_wf_accum, (npix + 255) / 256, 256, 0, st, P);
         ++launches;
