@@ -1025,7 +1025,11 @@ __global__ void __launch_bounds__(128, 6) k_restir_init(WfParams P) {
 // W = sum w / (Z target_here(y)), Z = the sum of M over the combined reservoirs whose own
 // initial target p0 is positive at y (those that could have drawn y).  The wave holds whole
 // windows.
-__global__ void __launch_bounds__(128, 6) k_restir_spatial(WfParams P, uint32_t n) {
+// Bound by the latency of the neighbours' scattered surfaces and reservoirs; 4 blocks per SM keep
+// the next neighbour's in registers (1080p, 248 lights, 5 neighbours, both passes: 0.76 ms with
+// 6 blocks and nothing ahead, 0.76 with 5 or 6 and one ahead, which spill it, 0.64 with 4).
+constexpr int SPATIAL_BLOCKS = 4;
+__global__ void __launch_bounds__(128, SPATIAL_BLOCKS) k_restir_spatial(WfParams P, uint32_t n) {
     if (P.counters[C_TAIL]) return;
     const uint32_t sbase = wf_sample_base(P);
     const uint64_t seed = wf_seed(P);
@@ -1053,37 +1057,64 @@ __global__ void __launch_bounds__(128, 6) k_restir_spatial(WfParams P, uint32_t 
             float3 y = xyz(f0);
             uint32_t used[64];
             uint32_t n_used = 0;
-            for (uint32_t j = 0; j < P.restir_K; ++j) {
+            // one neighbour ahead: its surface and reservoir are loaded while this one's target
+            // is evaluated
+            struct Neighbour {
+                bool in;
+                uint32_t id;
+                float u, depth;
+                float4 n, a0, a1;
+            };
+            auto fetch = [&](uint32_t j, Neighbour& b) {
                 const uint4 r = philox4x32_10(make_uint4(p, s, RESTIR_SPATIAL, j), k0, k1);
                 const int dx = (int)(((uint64_t)r.x * side) >> 32) - (int)P.restir_R;
                 const int dy = (int)(((uint64_t)r.y * side) >> 32) - (int)P.restir_R;
-                const float u_sel = u24(r.z);
+                b.u = u24(r.z);
                 const int nx = (int)rx + dx, ny = (int)ry + dy;
-                if ((dx == 0 && dy == 0) || nx < 0 || ny < 0 || nx >= (int)P.cw || ny >= (int)ch) continue;
-                const uint32_t nid = base + (uint32_t)ny * P.cw + (uint32_t)nx;
-                if (__float_as_uint(P.rs_g1[nid].w) == PT_NO_HIT) continue;
-                const float4 ng0 = P.rs_g0[nid], nn = P.rs_gn[nid];
-                if (dot3(xyz(nn), g.n) < 0.9f || fabsf(ng0.w - g0.w) > 0.1f * g0.w) continue;
-                used[n_used++] = nid;
-                const float4 a0 = P.rs_i[2u * nid], a1 = P.rs_i[2u * nid + 1];
+                b.in = !((dx == 0 && dy == 0) || nx < 0 || ny < 0 || nx >= (int)P.cw || ny >= (int)ch);
+                if (!b.in) return;
+                b.id = base + (uint32_t)ny * P.cw + (uint32_t)nx;
+                b.in = __float_as_uint(P.rs_g1[b.id].w) != PT_NO_HIT;
+                b.depth = P.rs_g0[b.id].w;      // unset where there is no surface
+                b.n = P.rs_gn[b.id];
+                b.a0 = P.rs_i[2u * b.id];
+                b.a1 = P.rs_i[2u * b.id + 1];
+            };
+            Neighbour next;
+            if (P.restir_K) fetch(0, next);
+            for (uint32_t j = 0; j < P.restir_K; ++j) {
+                const Neighbour b = next;
+                if (j + 1 < P.restir_K) fetch(j + 1, next);
+                if (!b.in) continue;
+                if (dot3(xyz(b.n), g.n) < 0.9f || fabsf(b.depth - g0.w) > 0.1f * g0.w) continue;
+                used[n_used++] = b.id;
                 float3 c, ld;
-                const float ph = restir_target(P.S, g.x, g.tt, g.bb, g.n, g.C, g.wo, __float_as_int(a0.w), xyz(a0), c, ld);
-                const float w = ph * a1.x * a1.y;
+                const float ph = restir_target(P.S, g.x, g.tt, g.bb, g.n, g.C, g.wo, __float_as_int(b.a0.w), xyz(b.a0), c, ld);
+                const float w = ph * b.a1.x * b.a1.y;
                 if (!(w > 0.0f)) continue;
                 wsum += w;
-                if (u_sel * wsum < w) {
-                    light = __float_as_int(a0.w);
-                    y = xyz(a0);
+                if (b.u * wsum < w) {
+                    light = __float_as_int(b.a0.w);
+                    y = xyz(b.a0);
                 }
             }
             float3 c, ld;
             const float ph = restir_target(P.S, g.x, g.tt, g.bb, g.n, g.C, g.wo, light, y, c, ld);
             float Z = restir_target0(P.S, g.x, g.n, transmits, light, y) > 0.0f ? Mq : 0.0f;
-            for (uint32_t u = 0; u < n_used; ++u) {
+            float4 ux = make_float4(0, 0, 0, 0), un = ux;
+            float um = 0.0f;
+            auto fetch_used = [&](uint32_t u) {
                 const uint32_t nid = used[u];
-                const float4 nn = P.rs_gn[nid];
-                if (restir_target0(P.S, xyz(P.rs_g0[nid]), xyz(nn), nn.w != 0.0f, light, y) > 0.0f)
-                    Z += P.rs_i[2u * nid + 1].y;
+                ux = P.rs_g0[nid];
+                un = P.rs_gn[nid];
+                um = P.rs_i[2u * nid + 1].y;
+            };
+            if (n_used) fetch_used(0);
+            for (uint32_t u = 0; u < n_used; ++u) {
+                const float4 x = ux, nn = un;
+                const float m = um;
+                if (u + 1 < n_used) fetch_used(u + 1);
+                if (restir_target0(P.S, xyz(x), xyz(nn), nn.w != 0.0f, light, y) > 0.0f) Z += m;
             }
             f0 = make_float4(y.x, y.y, y.z, __int_as_float(light));
             f1 = make_float4((ph > 0.0f && Z > 0.0f) ? wsum / (Z * ph) : 0.0f, Z, ph, 0.0f);
@@ -1884,7 +1915,7 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                     if (restir && k == 0) {
                         e = begin(PT_K_RESTIR);
                         PT_LAUNCH(k_restir_init, sms * 6, 128, 0, st, P);
-                        PT_LAUNCH(k_restir_spatial, sms * 6, 128, 0, st, P, n);
+                        PT_LAUNCH(k_restir_spatial, sms * SPATIAL_BLOCKS, 128, 0, st, P, n);
                         end(e);
                         launches += 2;
                     }
