@@ -279,10 +279,12 @@ __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const __half* p) {
 }
 
 // Fused cache inference: encoding and MLP of 16 queries per warp, the 64-wide input built in
-// a shared-memory tile (never written to HBM).  Lane j encodes level j % 16 of queries
-// 2r + j / 16 (r = 0..7): its level's resolution and table stay in registers and it issues
-// its 64 corner gathers back to back.  The tile then feeds the same tensor-core layers as
-// k_mlp_forward, with the A fragments read by ldmatrix.
+// a shared-memory tile (never written to HBM).  Lanes 2l and 2l + 1 encode level l of queries
+// 2r and 2r + 1 (r = 0..7): each gathers one x side of both queries' cells, so the two corners
+// along x, which lie in one 32-byte sector 7 times in 8, are one access of the pair, and the
+// values are exchanged and summed in corner order.  Bound by the L2 sectors of the fine levels
+// (1,000,003 random queries: 437 us with a whole cell per lane, 426 in pairs).  The tile then
+// feeds the same tensor-core layers as k_mlp_forward, with the A fragments read by ldmatrix.
 // 512 threads share one copy of the weights in shared memory (the copy, not the registers,
 // limited 128-thread blocks to 4 per SM); two blocks of sixteen warps fit per SM (64
 // registers, no spills)
@@ -297,33 +299,55 @@ __global__ void __launch_bounds__(INFER_THREADS, 2) k_nrc_infer(GridDesc G, cons
     const uint32_t n = rc.get();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     __half* X = sx[warp];
-    const uint32_t l = lane & 15;
+    const uint32_t l = lane >> 1, side = lane & 1;
     const bool grid_lane = l < G.L;
     const uint32_t res = grid_lane ? G.res[l] : 1u;
     const __half2* tab = reinterpret_cast<const __half2*>(G.table) + (size_t)l * G.T;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; tile * 16 < n; tile += warps) {
         const uint32_t r0 = tile * 16;
-        // grid features: columns 2l, 2l + 1 of rows 2r + lane / 16
+        // grid features, columns 2l, 2l + 1: rows 2r and 2r + 1 by the lane pair of level l
 #pragma unroll
         for (int r = 0; r < 8; ++r) {
-            const uint32_t row = 2 * r + (lane >> 4);
-            const uint32_t q = r0 + row;
+            const uint32_t row = 2 * r + side;
             float f0 = 0.0f, f1 = 0.0f;
-            if (grid_lane && q < n) {
-                const float3 p = pos01(G, queries + (size_t)QSTRIDE * q);
-                uint32_t cx, cy, cz;
-                float rx, ry, rz;
-                grid_cell(p, res, cx, cy, cz, rx, ry, rz);
+            float rx = 0.0f, ry = 0.0f, rz = 0.0f;
+            __half2 own[4], give[4];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint32_t ox = c & 1, oy = (c >> 1) & 1, oz = (c >> 2) & 1;
-                    const float w = (ox ? rx : 1.0f - rx) * (oy ? ry : 1.0f - ry) * (oz ? rz : 1.0f - rz);
-                    const float2 v = __half22float2(tab[corner_index(cx + ox, cy + oy, cz + oz, res, G.T)]);
+            for (uint32_t k = 0; k < 4; ++k) own[k] = give[k] = __half2();
+            if (grid_lane) {
+                // this lane's x side of both rows' cells
+#pragma unroll
+                for (uint32_t h = 0; h < 2; ++h) {
+                    const float3 p = pos01(G, queries + (size_t)QSTRIDE * min(r0 + 2 * r + h, n - 1u));
+                    uint32_t cx, cy, cz;
+                    float fx, fy, fz;
+                    grid_cell(p, res, cx, cy, cz, fx, fy, fz);
+                    const bool mine = h == side;
+                    if (mine) { rx = fx; ry = fy; rz = fz; }
+#pragma unroll
+                    for (uint32_t k = 0; k < 4; ++k) {
+                        const __half2 v = tab[corner_index(cx + side, cy + (k & 1u), cz + (k >> 1), res, G.T)];
+                        if (mine) own[k] = v;
+                        else give[k] = v;
+                    }
+                }
+            }
+            // the partner's side of this lane's row, then the corners in order
+#pragma unroll
+            for (uint32_t k = 0; k < 4; ++k) {
+                uint32_t u = *reinterpret_cast<uint32_t*>(&give[k]);
+                u = __shfl_xor_sync(0xffffffffu, u, 1);
+                const __half2 other = *reinterpret_cast<__half2*>(&u);
+#pragma unroll
+                for (uint32_t ox = 0; ox < 2; ++ox) {
+                    const float w = (ox ? rx : 1.0f - rx) * ((k & 1u) ? ry : 1.0f - ry) * ((k >> 1) ? rz : 1.0f - rz);
+                    const float2 v = __half22float2(ox == side ? own[k] : other);
                     f0 += w * v.x;
                     f1 += w * v.y;
                 }
             }
+            if (r0 + row >= n) f0 = f1 = 0.0f;
             if (grid_lane) *reinterpret_cast<__half2*>(X + row * SROW + 2 * l) = __floats2half2_rn(f0, f1);
         }
         // the other 64 - 2L columns: direction, normal, roughness, a constant 1, zeros
