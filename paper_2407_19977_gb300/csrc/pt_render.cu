@@ -498,8 +498,6 @@ __global__ void k_wf_raygen(WfParams P) {
     camera_ray_ps(P.cam, px, py, p, s, (uint32_t)seed, (uint32_t)(seed >> 32), o, d);
     P.ray_o[0][t] = make_float4(o.x, o.y, o.z, 0.0f);
     P.ray_d[0][t] = make_float4(d.x, d.y, d.z, __uint_as_float(id));
-    P.beta[id] = make_float4(1.0f, 1.0f, 1.0f, -1.0f);
-    P.radiance[id] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (P.nrc_on) {
         uint32_t aux = 0;
         if (P.max_train && u24(philox4x32_10(make_uint4(p, s, 0u, NRC_DIM_TRAIN >> 2), (uint32_t)seed,
@@ -1124,6 +1122,18 @@ __global__ void __launch_bounds__(128, SPATIAL_BLOCKS) k_restir_spatial(WfParams
     }
 }
 
+// State of path id at vertex k.  At the first vertex it is known: throughput 1, no pdf, no
+// radiance.  Neither written by the ray generation nor read back there, 64 bytes a path (1080p
+// CAD step 6.41 -> 6.39 ms, cached frame 0.928 -> 0.917).  In a merged batch the radiance's w word carries the
+// path's segment from the start.
+__device__ __forceinline__ float4 path_beta(const WfParams& P, uint32_t id, uint32_t k) {
+    return k == 0 ? make_float4(1.0f, 1.0f, 1.0f, -1.0f) : P.beta[id];
+}
+template <bool MULTI>
+__device__ __forceinline__ float4 path_radiance(const WfParams& P, uint32_t id, uint32_t k) {
+    return k == 0 && !MULTI ? make_float4(0.0f, 0.0f, 0.0f, 0.0f) : P.radiance[id];
+}
+
 // 16 bytes from global to shared memory without a register
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -1184,8 +1194,8 @@ __global__ void __launch_bounds__(128, shade_blocks(RIS, MULTI)) k_wf_shade(WfPa
             id = __float_as_uint(rd.w);
             HitRec h;
             h.t = hh.x; h.u = hh.y; h.v = hh.z; h.tri = __float_as_uint(hh.w);
-            b4 = P.beta[id];
-            const float4 L4 = P.radiance[id];
+            b4 = path_beta(P, id, k);
+            const float4 L4 = path_radiance<MULTI>(P, id, k);
             PathState ps;
             ps.beta = xyz(b4);
             ps.prev_pdf = b4.w;
@@ -1408,8 +1418,8 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
         const float4 ro = P.ray_o[in_q][i], rd = P.ray_d[in_q][i];
         const uint32_t id = __float_as_uint(rd.w);
-        const float4 b4 = P.beta[id];
-        const float4 L4 = P.radiance[id];
+        const float4 b4 = path_beta(P, id, k0);
+        const float4 L4 = path_radiance<MULTI>(P, id, k0);
         PathState ps;
         ps.beta = xyz(b4);
         ps.prev_pdf = b4.w;
@@ -1509,7 +1519,6 @@ __global__ void k_wfm_raygen(WfParams P, uint32_t n_paths) {
     camera_ray_ps(J.cam, px, py, p, s, (uint32_t)J.seed, (uint32_t)(J.seed >> 32), o, d);
     P.ray_o[0][id] = make_float4(o.x, o.y, o.z, __uint_as_float(g.job));
     P.ray_d[0][id] = make_float4(d.x, d.y, d.z, __uint_as_float(id));
-    P.beta[id] = make_float4(1.0f, 1.0f, 1.0f, -1.0f);
     P.radiance[id] = make_float4(0.0f, 0.0f, 0.0f, __uint_as_float(si));
     if (id == 0) atomicAdd(&P.stats[ST_PATHS], (unsigned long long)n_paths);
 }
@@ -1592,39 +1601,45 @@ __global__ void k_wf_accum(WfParams P) {
 }
 
 pt_status pt_free_wave(WaveBuffers& w) {
-    void* ps[] = {w.ray_o[0], w.ray_o[1], w.ray_d[0], w.ray_d[1], w.hit, w.beta, w.radiance,
-                  w.sh_o, w.sh_d, w.sh_c, w.perm, w.keys, w.counters, w.aux, w.nrc_q, w.nrc_out,
-                  w.nrc_counters, w.train_rec, w.train_nv, w.train_id, w.train_samples,
-                  w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
+    void* ps[] = {w.block, w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id,
+                  w.train_samples, w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
     for (void* p : ps)
         if (p) cudaFree(p);
     w = WaveBuffers();
     return PT_OK;
 }
 
+constexpr size_t WAVE_F4 = 10;   // float4 arrays per path: 2 x ray o/d, hit, beta, radiance, 3 x shadow
+
+static size_t wave_bytes(size_t paths) {
+    return paths * (WAVE_F4 * sizeof(float4) + 2 * sizeof(uint32_t)) + (C_BUCKETS + MAX_SORT_KEYS) * sizeof(uint32_t);
+}
+
+// carves a block of wave_bytes(c) bytes into the buffers of a wave of c paths
+static void carve_wave(WaveBuffers& w, void* block, size_t c) {
+    float4* f4 = reinterpret_cast<float4*>(block);
+    w.ray_o[0] = f4 + 0 * c; w.ray_o[1] = f4 + 1 * c;
+    w.ray_d[0] = f4 + 2 * c; w.ray_d[1] = f4 + 3 * c;
+    w.hit = f4 + 4 * c; w.beta = f4 + 5 * c; w.radiance = f4 + 6 * c;
+    w.sh_o = f4 + 7 * c; w.sh_d = f4 + 8 * c; w.sh_c = f4 + 9 * c;
+    uint32_t* u = reinterpret_cast<uint32_t*>(f4 + WAVE_F4 * c);
+    w.perm = u; w.keys = u + c; w.counters = u + 2 * c;
+    w.capacity = (uint32_t)c;
+    w.bytes = wave_bytes(c);
+}
+
+// one allocation for all of a wave's buffers (13 of them took 0.45 ms of a scene's first frame)
 static pt_status ensure_wave(WaveBuffers& w, uint32_t capacity) {
     if (w.capacity >= capacity) return PT_OK;
     pt_free_wave(w);
-    const size_t c = capacity;
-    float4** f4[] = {&w.ray_o[0], &w.ray_o[1], &w.ray_d[0], &w.ray_d[1], &w.hit, &w.beta, &w.radiance,
-                     &w.sh_o, &w.sh_d, &w.sh_c};
-    for (float4** p : f4) {
-        cudaError_t e = cudaMalloc((void**)p, c * sizeof(float4));
-        if (e != cudaSuccess) {
-            pt_free_wave(w);
-            pt_set_error(std::string("wavefront buffers: ") + cudaGetErrorString(e));
-            return PT_ERR_OOM;
-        }
-    }
-    if (cudaMalloc(&w.perm, c * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&w.keys, c * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMalloc(&w.counters, (C_BUCKETS + MAX_SORT_KEYS) * sizeof(uint32_t)) != cudaSuccess) {
-        pt_free_wave(w);
-        pt_set_error("wavefront buffers: out of memory");
+    void* block = nullptr;
+    const cudaError_t e = cudaMalloc(&block, wave_bytes(capacity));
+    if (e != cudaSuccess) {
+        pt_set_error(std::string("wavefront buffers: ") + cudaGetErrorString(e));
         return PT_ERR_OOM;
     }
-    w.capacity = capacity;
-    w.bytes = c * (10 * sizeof(float4) + 2 * sizeof(uint32_t));
+    carve_wave(w, block, capacity);
+    w.block = block;
     return PT_OK;
 }
 
@@ -2033,10 +2048,10 @@ static DJob make_job(pt_scene* s, const pt_camera& cam, uint32_t x0, uint32_t y0
 // many.  The path kernel is one launch but keeps a lane for a path to its end, so it loses once
 // there are paths to refill the lanes with.  Measured, path kernel against wavefront in ms, at
 // 65,536 / 131,072 / 160,000 / 320,000 / 524,288 paths: Cornell box 0.18 / 0.32 / 0.38 / 0.75 /
-// 1.23 against 0.33 / 0.34 / 0.38 / 0.50 / 0.65, 50k-triangle CAD model 0.62 / 0.82 / 0.98 /
-// 1.55 / 2.38 against 0.78 / 0.96 / 1.08 / 1.24 / 1.52, glass scene 0.50 / 0.69 / 0.77 / 1.31 /
-// 2.05 against 0.76 / 0.92 / 0.97 / 1.20 / 1.44.
-constexpr uint64_t AUTO_WAVE_PATHS = 1u << 18;
+// 1.22 against 0.27 / 0.29 / 0.32 / 0.43 / 0.58, 50k-triangle CAD model 0.63 / 0.83 / 0.95 /
+// 1.55 / 2.39 against 0.69 / 0.74 / 0.85 / 0.98 / 1.21, glass scene 0.51 / 0.70 / 0.75 / 1.31 /
+// 2.03 against 0.70 / 0.77 / 0.80 / 0.96 / 1.17.
+constexpr uint64_t AUTO_WAVE_PATHS = 1u << 17;
 
 static uint32_t auto_mode(const pt_render_opts& o, uint32_t npix, uint32_t spp, cudaStream_t st) {
     if (o.nrc) return PT_MODE_WAVEFRONT;
@@ -2489,9 +2504,8 @@ extern "C" pt_status pt_render_batch(const pt_job* jobs, uint32_t n_jobs, const 
 // queue, the shadow queue, the fetch heads and the sort buckets) and initialise every path
 // slot they read, so stale contents from an earlier call are never used.
 constexpr uint32_t NOALLOC_MAX_PATHS = 16384;
-constexpr size_t NOALLOC_F4 = 10;   // float4 arrays per path: 2 x ray o/d, hit, beta, radiance, 3 x shadow
 constexpr size_t NOALLOC_BYTES =
-    (size_t)NOALLOC_MAX_PATHS * (NOALLOC_F4 * sizeof(float4) + 2 * sizeof(uint32_t)) +
+    (size_t)NOALLOC_MAX_PATHS * (WAVE_F4 * sizeof(float4) + 2 * sizeof(uint32_t)) +
     (C_BUCKETS + MAX_SORT_KEYS) * sizeof(uint32_t);
 static __device__ __align__(256) unsigned char g_noalloc_scratch[NOALLOC_BYTES];
 
@@ -2540,17 +2554,8 @@ extern "C" pt_status pt_render_noalloc(pt_scene* s, const pt_camera* camera, uin
     if (r != PT_OK) return r;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     s->last_stream = st;
-    // carve the fixed array into the wavefront buffers
-    const size_t c = NOALLOC_MAX_PATHS;
-    float4* f4 = reinterpret_cast<float4*>(base);
     WaveBuffers w;
-    w.capacity = NOALLOC_MAX_PATHS;
-    w.ray_o[0] = f4 + 0 * c; w.ray_o[1] = f4 + 1 * c;
-    w.ray_d[0] = f4 + 2 * c; w.ray_d[1] = f4 + 3 * c;
-    w.hit = f4 + 4 * c; w.beta = f4 + 5 * c; w.radiance = f4 + 6 * c;
-    w.sh_o = f4 + 7 * c; w.sh_d = f4 + 8 * c; w.sh_c = f4 + 9 * c;
-    uint32_t* u = reinterpret_cast<uint32_t*>(f4 + NOALLOC_F4 * c);
-    w.perm = u; w.keys = u + c; w.counters = u + 2 * c;
+    carve_wave(w, base, NOALLOC_MAX_PATHS);
     const uint32_t npix = acc->width * acc->height;
     const uint32_t samp_per_wave = std::max(1u, std::min(spp, NOALLOC_MAX_PATHS / npix));
     const bool sort = o.sort_by_material == 1 || (o.sort_by_material < 0 && s->n_mats + 2 <= MAX_SORT_KEYS && s->n_mats > 1);
