@@ -1,4 +1,5 @@
 // pt_api.cu -- C-ABI entry points: scene setup and teardown, diagnostics, statistics.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -150,6 +151,23 @@ static bool material_ok(const pt_openpbr& m, std::string& why) {
     return true;
 }
 
+// Host arrays where there is no device to check them on: 0, or the same bits as the device checks
+// set (1 vertex, 2 index, 4 material id, 8 environment texel).
+static uint32_t check_host_arrays(const float* v, uint64_t nv3, uint32_t n_vertices, const uint32_t* idx,
+                                  const uint32_t* mid, uint64_t nt, uint32_t n_mats, const float* env, uint64_t ne) {
+    uint32_t bad = 0;
+    for (uint64_t i = 0; v && i < nv3; ++i) bad |= std::isfinite(v[i]) ? 0u : 1u;
+    for (uint64_t i = 0; i < 3 * nt; ++i) bad |= idx[i] < n_vertices ? 0u : 2u;
+    for (uint64_t i = 0; i < nt; ++i) bad |= mid[i] < n_mats ? 0u : 4u;
+    for (uint64_t i = 0; env && i < ne; ++i) bad |= std::isfinite(env[i]) && env[i] >= 0.0f ? 0u : 8u;
+    return bad;
+}
+static pt_status bad_arrays(uint32_t bad) {
+    pt_set_error(bad & 1 ? "non-finite vertex" : bad & 2 ? "vertex index out of range"
+                 : bad & 4 ? "material id out of range" : "bad env texel");
+    return PT_ERR_INVALID_ARG;
+}
+
 static void free_scene(pt_scene* s) {
     if (!s) return;
     void* ptrs[] = {s->d_vertices, s->d_indices, s->d_matids, s->d_tris_raw, s->d_tris, s->d_nodes,
@@ -192,10 +210,17 @@ extern "C" pt_status pt_scene_create(const float* vertices, uint32_t n_vertices,
         const double cz = (double)q[3] * q[7] - (double)q[4] * q[6];
         PT_CHECK_ARG(cx * cx + cy * cy + cz * cz > 0.0, "degenerate quad light");
     }
-    // vertices without triangles are never uploaded
-    if (!inputs_on_device && n_triangles == 0 && vertices)
-        for (uint64_t i = 0; i < (uint64_t)n_vertices * 3; ++i)
-            PT_CHECK_ARG(std::isfinite(vertices[i]), "non-finite vertex");
+    // The arrays are checked on the device, host inputs too (host loops over a 1.07M-triangle
+    // model took 1.4 to 2.5 ms).  Bad host arrays are bad without a device as well; and vertices
+    // without triangles are never uploaded.
+    int n_devices = 0;
+    const bool no_device = cudaGetDeviceCount(&n_devices) != cudaSuccess || n_devices == 0;
+    if (!inputs_on_device && (no_device || n_triangles == 0)) {
+        cudaGetLastError();
+        const uint32_t bad = check_host_arrays(vertices, (uint64_t)n_vertices * 3, n_vertices, indices, material_ids,
+                                               n_triangles, n_materials, env_rgb, (uint64_t)env_w * env_h * 3);
+        if (bad) return bad_arrays(bad);
+    }
     cudaStream_t st = (cudaStream_t)cuda_stream;
     pt_scene* s = new pt_scene();
     s->serial = pt_next_serial();
@@ -254,8 +279,6 @@ extern "C" pt_status pt_scene_create(const float* vertices, uint32_t n_vertices,
     uint32_t* d_scratch = nullptr;
     TRY(cudaMalloc(&d_scratch, kScratchWords * sizeof(uint32_t)));
     TRY(cudaMemsetAsync(d_scratch, 0, kScratchWords * sizeof(uint32_t), st));
-    // the arrays are checked on the device, host inputs too (a host loop over 1.07M triangles'
-    // arrays took 2.5 ms)
     if (n_triangles > 0)
         PT_LAUNCH(k_validate_vertices, (uint32_t)(((uint64_t)n_vertices * 3 + 255) / 256), 256, 0, st, s->d_vertices,
                   n_vertices * 3u, d_scratch + 8);
@@ -295,10 +318,8 @@ extern "C" pt_status pt_scene_create(const float* vertices, uint32_t n_vertices,
     cudaFree(d_scratch);
 #undef TRY
     if (bad) {
-        pt_set_error(bad & 1 ? "non-finite vertex" : bad & 2 ? "vertex index out of range"
-                     : bad & 4 ? "material id out of range" : "bad env texel");
         free_scene(s);
-        return PT_ERR_INVALID_ARG;
+        return bad_arrays(bad);
     }
     *out = s;
     return PT_OK;
