@@ -1730,17 +1730,28 @@ struct WfGraphKey {
     uint64_t nrc_serial;    // the radiance cache the launches read and train (0: none)
 };
 
+// whether calls on the stream are being captured (or cannot be asked because another is)
+static bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t spp, uint32_t max_depth, uint64_t seed,
                                   pt_accum* acc, const pt_render_opts& o, cudaStream_t user_st) {
     cudaStream_t st = user_st;   // the stream the wave loops below issue to (a capture stream while capturing)
     const uint32_t npix_total = acc->width * acc->height;
-    // automatic wave: 2^23 paths (1.4 GB of queues), or 2^21 where there is no room for that and
-    // in frames that train the cache (a wave is a training set).  Every pass of a wave ends with
+    // automatic wave: 2^23 paths (1.4 GB of queues), or 2^21 where there is no room for that, in
+    // frames that train the cache (a wave is a training set) and under stream capture, where the
+    // buffers of an earlier, smaller call cannot grow.  Every pass of a wave ends with
     // the chip waiting for its longest rays, so few large waves beat many small ones: 2^21 /
     // 2^22 / 2^23 / 2^24 paths a wave, 512 x 512 still of 25 samples 10.12 / 7.93 / 6.84 / 6.84
     // ms, glass scene at 1917 x 1079 and 2 samples 5.85 / 4.20 / 4.21 / 4.23.
     constexpr uint32_t LARGE_WAVE = 1u << 23, SMALL_WAVE = 1u << 21;
-    const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train);
+    const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train) && !capturing(user_st);
     uint32_t cap = std::max(o.wave_paths ? o.wave_paths : large ? LARGE_WAVE : SMALL_WAVE, 32u);
     // waves hold whole samples of a pixel range: pixel chunk <= cap, then samples per wave;
     // with ReSTIR the chunk is the whole window (the spatial pass reads any pixel of it)
@@ -2064,12 +2075,7 @@ static uint32_t auto_mode(const pt_render_opts& o, uint32_t npix, uint32_t spp, 
     }
     if (few) return PT_MODE_MEGAKERNEL;
     // a small frame that is being captured allocates nothing: the path kernel needs no buffers
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return PT_MODE_MEGAKERNEL;
-    }
-    return cap == cudaStreamCaptureStatusNone ? PT_MODE_WAVEFRONT : PT_MODE_MEGAKERNEL;
+    return capturing(st) ? PT_MODE_MEGAKERNEL : PT_MODE_WAVEFRONT;
 }
 
 extern "C" pt_status pt_render(pt_scene* s, const pt_camera* camera, uint32_t spp, uint32_t max_depth, uint64_t seed,

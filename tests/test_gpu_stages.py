@@ -27,3 +27,36 @@ def test_staged_passes_equal_path_kernel(scene, crop, spp):
             assert torch.equal(x, y)
     st = g.stats()
     assert st["error_flags"] == 0 and bool((out[0][0] >= 0).all())
+
+
+@pytest.mark.parametrize("side,spp", [(64, 31), (64, 32), (181, 4), (255, 3)])
+def test_auto_picks_either_route_with_the_same_sums(side, spp):
+    """Frames on both sides of AUTO's line (131,072 paths), eager and under stream capture, where
+    a small frame must not allocate: the sums of both explicit modes, bit for bit."""
+    from paper_2407_19977_gb300 import api, native as N, scenes
+    sc = scenes.cornell_box(seed=2, width=side, height=side, max_depth=4)
+    g = api.Scene(sc)
+    acc = api.Accum(side, side)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        g.render(spp, seed=5, accum=acc)
+    graph.replay()
+    want = g.render(spp, seed=5, mode=N.PT_MODE_WAVEFRONT)
+    for a in (acc, g.render(spp, seed=5), g.render(spp, seed=5, mode=N.PT_MODE_MEGAKERNEL)):
+        assert torch.equal(a.sum, want.sum) and torch.equal(a.comp, want.comp)
+
+
+def test_capture_after_a_smaller_call():
+    """A captured call of more samples than the call that sized the wave's buffers runs in waves
+    that fit them."""
+    from paper_2407_19977_gb300 import api, scenes
+    sc = scenes.cornell_box(seed=2, width=1536, height=1400, max_depth=3)     # above 2^21 pixels
+    g = api.Scene(sc)
+    g.render(1, seed=5)
+    acc = api.Accum(1536, 1400)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        g.render(3, seed=5, accum=acc)
+    graph.replay()
+    want = g.render(3, seed=5)
+    assert torch.equal(acc.sum, want.sum) and torch.equal(acc.comp, want.comp)
