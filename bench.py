@@ -583,7 +583,7 @@ def run_ours(args, world, rank, local):
         "e2e": {"value": e2e_val, "unit": "Mrays/s", "h2d_bytes_per_step": 48 + 8,
                 "d2h_bytes_per_step": W * H * 3 * 4,
                 "copies": "each frame's image to pinned host memory, double-buffered on a copy stream"},
-        "roofline": {"bound": "alu", "kernel": "k_wf_trace (closest hit)",
+        "roofline": {"bound": "alu", "kernel": "k_wf_rays (closest hit)",
                      "achieved": achieved_gops, "peak": alu_peak, "unit": "GOP/s",
                      "frac": achieved_gops / alu_peak if achieved_gops else None,
                      "traffic": traffic,
