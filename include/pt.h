@@ -422,8 +422,8 @@ pt_status pt_render_batch(const pt_job* jobs, uint32_t n_jobs, const pt_batch_op
  * warm-up frame) of `spp` samples per candidate into a scratch accumulator of camera->width x
  * height and times them with CUDA events on the stream; candidates: wavefront with material
  * sort off/on x tail limit (off, automatic, a quarter, four times) x wave size (2^20 .. 2^23
- * paths, as far as the call needs them), graph replay on; megakernel with 32, 64, 128 pixels
- * per work item; then the winner's traversal passes one ray per lane or per 8-lane group, and a
+ * paths, as far as the call needs them), graph replay on; the path kernel with 32, 64, 128 threads
+ * per block; then the winner's traversal passes one ray per lane or per 8-lane group, and a
  * wavefront winner with a tail limit with tail_bounce 3, 4, 5 and 6.  With
  * PT_TUNE_BVH it first rebuilds the BVH with both builders and leaf sizes 1..4 at width 8, then
  * the fastest of those at widths 4 and 6 (pt_bvh_opts.max_width), and keeps the fastest tree.  The winner goes to *best (and ms per frame to
