@@ -777,9 +777,9 @@ __device__ __forceinline__ void closest_init(const DScene& S, float3 o, float3 d
 // check inside the loop (at most 7 a node, so no write leaves the array) and the overflow of
 // the PT_STACK entries the traversal may use is checked once after it.
 // BRANCHLESS selects the form of the child loop; both push the same children in the same
-// order.  The per-bounce closest-hit kernel keeps the branching form (a slot that misses
-// skips the push logic): on the 1080p CAD frame it measured 3.68 against 3.99 ms a step.  The
-// out-of-line traversal that the tail kernel and the megakernel call takes the form without
+// order.  The branching form (a slot that misses skips the push logic) suits coherent rays: the
+// feature pass takes it (1080p preview 3.34 -> 3.28 ms; the per-bounce passes, which took it
+// before they went in stages, 3.99 -> 3.68).  The out-of-line traversal that the tail kernel and the megakernel call takes the form without
 // branches, which measured faster there (tail kernel 0.49 -> 0.41 ms a step on the same
 // frame, 1.45 -> 1.19 ms on the 5.2M-triangle scene), where the lanes of a warp are at
 // different bounces and stages.

@@ -2,13 +2,13 @@
 // Sec. 5.1.4 progressive averaging).
 //
 // Two executions of the same per-vertex code (shade_vertex in pt_device.cuh):
-//  * megakernel: a persistent grid; warps pop (job, pixel tile) items from a work queue in
-//    device memory, each lane traces its pixel's samples in order and Kahan-accumulates.
-//    One launch also serves a batch of many scenes (pt_render_batch).
-//  * wavefront: one kernel per stage and bounce over queues in HBM: raygen -> closest hit
-//    (persistent, queue-fetching) -> optional sort of the queue by material -> shade
-//    (appends next rays and shadow rays with warp-aggregated atomics) -> shadow any-hit
-//    -> per-pixel Kahan accumulation in sample order.
+//  * one kernel: a thread per path, several samples of a pixel side by side, added in sample
+//    order (pt_render); for a batch of many scenes (pt_render_batch) a persistent grid whose
+//    warps pop (job, pixel tile) items from a work queue, a lane per pixel.
+//  * wavefront: kernels over queues in HBM: raygen -> per bounce: rays (closest hits, and the
+//    shadow rays of the bounce before) -> tail, if few paths are left -> optional sort of the
+//    queue by material -> shade (appends next rays and shadow rays with warp-aggregated
+//    atomics) -> per-pixel Kahan accumulation in sample order.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -1400,7 +1400,7 @@ __global__ void __launch_bounds__(128) k_wf_shadow_coop(WfParams P) {
 // stage and bounce.  This kernel takes the remaining queue instead, its rays just traced, and
 // carries each path to its end in one thread: closest hit, shade_vertex_h (the same per-vertex code and random
 // numbers as k_wf_shade), then the shadow ray, whose contribution is added after the vertex's
-// own terms exactly as k_wf_shadow adds it.  It appends nothing, so the later per-bounce
+// own terms exactly as shadow_queue adds it.  It appends nothing, so the later per-bounce
 // launches of the wave find empty queues (and C_TAIL makes the rest of this bounce skip).
 template <bool NRC, bool COUNT, bool RIS, bool FUZZ = true, bool MULTI = false>
 __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32_t k0, uint32_t limit) {
