@@ -1343,6 +1343,73 @@ static __device__ __noinline__ bool trace_any(const DScene& S, float3 o, float3 
     return trace_any_t<false>(S, o, d, tmax, tc);
 }
 
+// The same for the tail kernel, whose paths are at different vertices: the node visits of the
+// staged passes (loops over the children that are hit, where the loops above have a body per
+// slot).  Same visits in the same order.  Glass scene's tail 0.91 -> 0.86 ms (the frame 3.65 ->
+// 3.51), 1080p preview with features and denoiser 3.03 -> 3.00; but a 64 x 64 Cornell frame in
+// the path kernel, where a warp's rays are alike, 0.20 -> 0.23, so that keeps the loops above.
+static __device__ __noinline__ void tail_closest(const DScene& S, float3 o, float3 d, float tmax, HitRec& h) {
+    LaneRay r;
+    uint2 stack[PT_STACK + PT_STACK_SLACK];
+    TravCount tc = {0, 0, 0};
+    lane_ray_init(o, d, (uint32_t)S.n_nodes, r);
+    h.t = tmax;
+    h.tri = PT_NO_HIT;
+    h.u = h.v = 0.0f;
+    uint32_t best_orig = PT_NO_HIT;
+    for (;;) {
+        // more visits than nodes mean a malformed tree
+        if (r.budget-- <= 1u) {
+            if (S.n_nodes != 0) atomicOr(S.err, 4u);
+            h.tri = PT_NO_HIT;
+            return;
+        }
+        lane_closest_node<false>(S.nodes, r, h.t, stack, tc);
+        if (r.sp > PT_STACK) { atomicOr(S.err, 1u); return; }
+        for (; r.tri_mask; r.tri_mask &= r.tri_mask - 1u) {
+            const uint32_t ti = r.tri_base + (uint32_t)(__ffs(r.tri_mask) - 1);
+            const float4 a = __ldg(S.tris + 3u * ti), b = __ldg(S.tris + 3u * ti + 1), c = __ldg(S.tris + 3u * ti + 2);
+            float t, u, w;
+            if (tri_hit(r.wr, xyz(a), xyz(b), xyz(c), tmax, t, u, w)) {
+                const uint32_t orig = __float_as_uint(a.w);
+                if (t < h.t || (t == h.t && orig < best_orig)) {
+                    h.t = t; h.u = u; h.v = w; h.tri = ti; best_orig = orig;
+                }
+            }
+        }
+        while (!(r.near_t <= h.t)) {
+            if (r.sp == 0) return;
+            const uint2 e = stack[--r.sp];
+            r.node = e.x;
+            r.near_t = __uint_as_float(e.y);
+        }
+    }
+}
+static __device__ __noinline__ bool tail_any(const DScene& S, float3 o, float3 d, float tmax) {
+    LaneRay r;
+    uint32_t stack[PT_STACK + PT_STACK_SLACK];
+    TravCount tc = {0, 0, 0};
+    lane_ray_init(o, d, (uint32_t)S.n_nodes, r);
+    for (;;) {
+        if (r.budget-- <= 1u) {
+            if (S.n_nodes != 0) atomicOr(S.err, 4u);
+            return false;
+        }
+        lane_any_node<false>(S.nodes, r, tmax, stack, tc);
+        if (r.sp > PT_STACK) { atomicOr(S.err, 1u); return true; }
+        for (; r.tri_mask; r.tri_mask &= r.tri_mask - 1u) {
+            const uint32_t ti = r.tri_base + (uint32_t)(__ffs(r.tri_mask) - 1);
+            const float4 a = __ldg(S.tris + 3u * ti), b = __ldg(S.tris + 3u * ti + 1), c = __ldg(S.tris + 3u * ti + 2);
+            float t, u, w;
+            if (tri_hit(r.wr, xyz(a), xyz(b), xyz(c), tmax, t, u, w)) return true;
+        }
+        if (r.node == PT_NO_HIT) {
+            if (r.sp == 0) return false;
+            r.node = stack[--r.sp];
+        }
+    }
+}
+
 // ------------------------------------------------------------------ environment
 __device__ __forceinline__ void env_texel(const DScene& S, float3 d, int& x, int& y) {
     const float u = 0.5f + atan2f(d.x, -d.z) * (0.5f * PT_INV_PI_F);

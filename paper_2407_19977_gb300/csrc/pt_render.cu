@@ -1452,7 +1452,7 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
                 h.t = hh.x; h.u = h.v = 0.0f; h.tri = __float_as_uint(hh.w);
             } else {
                 if (COUNT) trace_closest_t<true, true>(S, o, d, __int_as_float(0x7f800000), h, tc);
-                else trace_closest(S, o, d, __int_as_float(0x7f800000), h);
+                else tail_closest(S, o, d, __int_as_float(0x7f800000), h);
                 n_ext++;
             }
             rng.k = k;
@@ -1465,7 +1465,7 @@ __global__ void __launch_bounds__(128, 4) k_wf_tail(WfParams P, int in_q, uint32
             if (so.has_shadow) {
                 n_sh++;
                 const bool occ = COUNT ? trace_any_t<true>(S, so.sh.o, so.sh.d, so.sh.tmax, sc)
-                                       : trace_any(S, so.sh.o, so.sh.d, so.sh.tmax);
+                                       : tail_any(S, so.sh.o, so.sh.d, so.sh.tmax);
                 if (!occ) {
                     ps.L.x += so.sh.contrib.x;
                     ps.L.y += so.sh.contrib.y;
