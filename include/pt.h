@@ -338,6 +338,10 @@ pt_status pt_bvh_build(pt_scene* scene, const pt_bvh_opts* opts, void* cuda_stre
  * closest hit, emission with MIS, next-event estimation to quads and the environment,
  * OpenPBR BSDF sample, Russian roulette, max_depth BSDF bounces, Kahan accumulation.
  * seed keys the Philox4x32-10 counter (pixel, sample, bounce, dim/4).
+ * Under stream capture (cuda_stream being captured by the caller) the call must fit the work
+ * buffers of an earlier call, or be one that needs none.  The captured graph may be replayed
+ * until the scene is rebuilt or destroyed: buffers it holds that a later, larger call replaces
+ * are kept until the scene is destroyed.
  * Errors: PT_ERR_NOT_BUILT, PT_ERR_INVALID_ARG (window outside the frame, NULL accum),
  * PT_ERR_OOM (work buffers), PT_ERR_CUDA. */
 pt_status pt_render(pt_scene* scene, const pt_camera* camera, uint32_t spp, uint32_t max_depth,

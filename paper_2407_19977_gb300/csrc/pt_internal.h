@@ -52,6 +52,11 @@ enum { ST_EXT = 0, ST_SHADOW = 1, ST_PATHS = 2, ST_NAN = 3, ST_RR = 4, ST_NRC = 
 // ---- wavefront workspace ---------------------------------------------------------------
 struct WaveBuffers {
     uint32_t capacity = 0;       // paths per wave
+    // a caller's stream capture has recorded addresses of these buffers: its graph may be
+    // replayed as long as the scene lives, so buffers that are replaced then go to `retired`
+    // (freed with the scene) instead of being freed
+    bool recorded = false;
+    std::vector<void*> retired;
     void* block = nullptr;       // the allocation that holds the buffers up to `counters`
     float4* ray_o[2] = {nullptr, nullptr};   // queue entries: origin (w unused)
     float4* ray_d[2] = {nullptr, nullptr};   // direction, w = path id bits

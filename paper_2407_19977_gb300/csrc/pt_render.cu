@@ -1600,11 +1600,27 @@ __global__ void k_wf_accum(WfParams P) {
     if (lane_id() == 0 && nan_cnt) atomicAdd(&P.stats[ST_NAN], nan_cnt);
 }
 
-pt_status pt_free_wave(WaveBuffers& w) {
+// a buffer that is replaced: freed, or kept for the graphs that may hold its address
+static void drop_buffer(WaveBuffers& w, void* p) {
+    if (!p) return;
+    if (w.recorded) w.retired.push_back(p);
+    else cudaFree(p);
+}
+
+// drops every buffer; what captures hold stays in `retired`
+static void reset_wave(WaveBuffers& w) {
     void* ps[] = {w.block, w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id,
                   w.train_samples, w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
-    for (void* p : ps)
-        if (p) cudaFree(p);
+    for (void* p : ps) drop_buffer(w, p);
+    std::vector<void*> kept;
+    kept.swap(w.retired);
+    w = WaveBuffers();
+    w.retired.swap(kept);
+}
+
+pt_status pt_free_wave(WaveBuffers& w) {
+    reset_wave(w);
+    for (void* p : w.retired) cudaFree(p);
     w = WaveBuffers();
     return PT_OK;
 }
@@ -1631,7 +1647,7 @@ static void carve_wave(WaveBuffers& w, void* block, size_t c) {
 // one allocation for all of a wave's buffers (13 of them took 0.45 ms of a scene's first frame)
 static pt_status ensure_wave(WaveBuffers& w, uint32_t capacity) {
     if (w.capacity >= capacity) return PT_OK;
-    pt_free_wave(w);
+    reset_wave(w);
     void* block = nullptr;
     const cudaError_t e = cudaMalloc(&block, wave_bytes(capacity));
     if (e != cudaSuccess) {
@@ -1649,8 +1665,7 @@ static pt_status ensure_nrc_buffers(WaveBuffers& w, uint32_t rec_per_path, uint3
     const uint32_t cap = w.capacity, slots = std::max(samples / 2, 1u);
     if (w.nrc_capacity >= cap && w.rec_per_path >= rec_per_path && w.sample_cap == samples) return PT_OK;
     void* ps[] = {w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id, w.train_samples};
-    for (void* q : ps)
-        if (q) cudaFree(q);
+    for (void* q : ps) drop_buffer(w, q);
     PT_CUDA_TRY(cudaMalloc(&w.aux, (size_t)cap * sizeof(uint32_t)));
     PT_CUDA_TRY(cudaMalloc(&w.nrc_q, (size_t)cap * 16 * sizeof(float)));
     PT_CUDA_TRY(cudaMalloc(&w.nrc_out, (size_t)cap * 4 * sizeof(float)));
@@ -1670,8 +1685,7 @@ static pt_status ensure_nrc_buffers(WaveBuffers& w, uint32_t rec_per_path, uint3
 static pt_status ensure_restir_buffers(WaveBuffers& w) {
     if (w.restir_capacity >= w.capacity) return PT_OK;
     void* ps[] = {w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
-    for (void* q : ps)
-        if (q) cudaFree(q);
+    for (void* q : ps) drop_buffer(w, q);
     w.rs_g0 = w.rs_g1 = w.rs_gn = w.rs_i = w.rs_f = nullptr;
     w.restir_capacity = 0;
     const size_t c = w.capacity;
@@ -1751,7 +1765,8 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
     // 2^22 / 2^23 / 2^24 paths a wave, 512 x 512 still of 25 samples 10.12 / 7.93 / 6.84 / 6.84
     // ms, glass scene at 1917 x 1079 and 2 samples 5.85 / 4.20 / 4.21 / 4.23.
     constexpr uint32_t LARGE_WAVE = 1u << 23, SMALL_WAVE = 1u << 21;
-    const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train) && !capturing(user_st);
+    const bool captured = capturing(user_st);
+    const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train) && !captured;
     uint32_t cap = std::max(o.wave_paths ? o.wave_paths : large ? LARGE_WAVE : SMALL_WAVE, 32u);
     // waves hold whole samples of a pixel range: pixel chunk <= cap, then samples per wave;
     // with ReSTIR the chunk is the whole window (the spatial pass reads any pixel of it)
@@ -1768,11 +1783,13 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
     pt_status r = buffers();
     if (r == PT_ERR_OOM && large) {
         cudaGetLastError();
-        pt_free_wave(w);
+        reset_wave(w);
         cap = SMALL_WAVE;
         r = buffers();
     }
     if (r != PT_OK) return r;
+    // from here on a caller's graph may hold the buffers' addresses
+    w.recorded = w.recorded || captured;
     const bool sort = o.sort_by_material == 1 || (o.sort_by_material < 0 && s->n_mats + 2 <= MAX_SORT_KEYS && s->n_mats > 1);
     const uint32_t n_keys = (sort && s->n_mats + 2 <= MAX_SORT_KEYS) ? s->n_mats + 2 : 0;
     wf_occupancy();
@@ -1987,8 +2004,8 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
         const cudaError_t ce = cudaStreamEndCapture(s->cap_stream, &g);
         st = user_st;
         // captured launches were recorded, not run: they count when the graph runs
-        const uint64_t captured = g_pt_launches.load() - global_before;
-        g_pt_launches.fetch_sub(captured);
+        const uint64_t recorded = g_pt_launches.load() - global_before;
+        g_pt_launches.fetch_sub(recorded);
         if (ir != PT_OK) {
             if (g) cudaGraphDestroy(g);
             return ir;
@@ -2006,9 +2023,9 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
         }
         s->wf_graph = ex;
         s->wf_key.assign(reinterpret_cast<const unsigned char*>(&key), reinterpret_cast<const unsigned char*>(&key) + sizeof(key));
-        s->wf_graph_launches = captured;
+        s->wf_graph_launches = recorded;
         PT_CUDA_TRY(cudaGraphLaunch(ex, user_st));
-        pt_count_launch(captured);
+        pt_count_launch(recorded);
     } else if (ir != PT_OK) {
         return ir;
     }
