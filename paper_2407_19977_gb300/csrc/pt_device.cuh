@@ -664,9 +664,11 @@ __device__ __forceinline__ NodeView load_node(const uint4* __restrict__ nodes, u
 // u = 2^-24: the reciprocal, subtraction and product in a (4 u |a|), b (3 u over at most
 // 255 |b|), the builder's one-rounding decode of the plane (u |plane/d| <= u (|a| + |o/d| +
 // 255 |b|)), the fma's result (u (|a| + 255 |b|)), c and c -+ e (2 u (|a| + 2^15 |b|)): at
-// most 4.8e-7 |a| + 4.1e-3 |b| + 6e-8 |o/d|, so the test stays conservative.  (A b or c that
-// overflows makes that axis's distances NaN, which the minimum and maximum ignore: the box is
-// then tested on the other axes only, which is conservative too.)
+// most 4.8e-7 |a| + 4.1e-3 |b| + 6e-8 |o/d|, so the test stays conservative.  The term in b is
+// taken from c, |b| <= 2^-15 (|c| + |a|): where 2^15 b overflows, c and with it e are infinite,
+// so that c - e is -inf or NaN and c + e is +inf or NaN, as they are for a or b infinite.  Either
+// way the minimum and maximum ignore that axis and the box is tested on the others only, which
+// is conservative too.
 struct NodeTest {
     float3 cn, cf, b;                              // c -/+ e, scale/d
     uint32_t nx0, nx1, ny0, ny1, nz0, nz1;         // near-plane byte words per axis
@@ -682,7 +684,7 @@ __device__ __forceinline__ void slab_terms(float p, float o, float inv, float sc
     const float a = __fmul_rn(__fsub_rn(p, o), inv);
     b = __fmul_rn(scale, inv);
     const float c = fmaf(-32768.0f, b, a);
-    const float e = fmaf(fabsf(b), 4.2e-3f, fmaf(fabsf(a), 6e-7f, fabsf(o * inv) * 3e-7f));
+    const float e = fmaf(fabsf(c), 4.2e-3f / 32768.0f, fmaf(fabsf(a), 7.3e-7f, fabsf(o * inv) * 3e-7f));
     cn = __fsub_rn(c, e);
     cf = __fadd_rn(c, e);
 }
