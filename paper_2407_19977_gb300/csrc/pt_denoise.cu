@@ -23,7 +23,9 @@ __global__ void k_features(DScene S, DCam cam, uint32_t x0, uint32_t y0, uint32_
     // a warp covers a compact 8 x 4 tile of the window, whose camera rays meet the same nodes, and
     // traces with the branching loop, which suits them (1080p preview with its features: 3.42 ms
     // with rows of 32 pixels, 3.34 in tiles, 3.28 with that loop)
-    const uint32_t tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31u, tw = (cw + 7u) / 8u;
+    // (the tile's index, not the thread's, which a thin window of many rows takes past 32 bits)
+    const uint32_t tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31u,
+                   tw = (cw + 7u) / 8u;
     const uint32_t wx = (tile % tw) * 8u + (lane & 7u), wy = (tile / tw) * 4u + (lane >> 3);
     if (wx >= cw || wy >= ch) return;
     const uint32_t i = wy * cw + wx;
@@ -52,9 +54,9 @@ __global__ void k_features(DScene S, DCam cam, uint32_t x0, uint32_t y0, uint32_
         hits += 1.0f;
     }
     const float inv = spp ? 1.0f / (float)spp : 0.0f;
-    out[3u * i] = make_float4(n_sum.x * inv, n_sum.y * inv, n_sum.z * inv, hits * inv);
-    out[3u * i + 1] = make_float4(x_sum.x * inv, x_sum.y * inv, x_sum.z * inv, 0.0f);
-    out[3u * i + 2] = make_float4(a_sum.x * inv, a_sum.y * inv, a_sum.z * inv, 0.0f);
+    out[3ull * i] = make_float4(n_sum.x * inv, n_sum.y * inv, n_sum.z * inv, hits * inv);
+    out[3ull * i + 1] = make_float4(x_sum.x * inv, x_sum.y * inv, x_sum.z * inv, 0.0f);
+    out[3ull * i + 2] = make_float4(a_sum.x * inv, a_sum.y * inv, a_sum.z * inv, 0.0f);
 }
 
 // ------------------------------------------------------------------ the regression
