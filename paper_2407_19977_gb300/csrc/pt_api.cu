@@ -30,8 +30,8 @@ __global__ void k_validate_vertices(const float* v, uint32_t n, uint32_t* bad) {
     if (i < n && !isfinite(v[i])) atomicOr(bad, 1u);
 }
 
-__global__ void k_validate_env(const float* env, uint32_t n, uint32_t* bad) {
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_validate_env(const float* env, uint64_t n, uint32_t* bad) {
+    const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
     if (i < n && (!isfinite(env[i]) || env[i] < 0.0f)) atomicOr(bad, 8u);
 }
 
@@ -286,7 +286,7 @@ extern "C" pt_status pt_scene_create(const float* vertices, uint32_t n_vertices,
         const size_t ne = (size_t)env_w * env_h * 3;
         TRY(cudaMalloc(&s->d_env, ne * sizeof(float)));
         TRY(cudaMemcpyAsync(s->d_env, env_rgb, ne * sizeof(float), kind, st));
-        PT_LAUNCH(k_validate_env, (uint32_t)((ne + 255) / 256), 256, 0, st, s->d_env, (uint32_t)ne, d_scratch + 8);
+        PT_LAUNCH(k_validate_env, (uint32_t)((ne + 255) / 256), 256, 0, st, s->d_env, (uint64_t)ne, d_scratch + 8);
         s->env_w = (int)env_w;
         s->env_h = (int)env_h;
     }

@@ -1,4 +1,4 @@
-"""Primary-hit features of windows of every shape."""
+"""Primary-hit features of windows of every shape, and inputs whose indices pass 32 bits."""
 import ctypes as C
 import dataclasses
 
@@ -42,3 +42,26 @@ def test_features_of_a_window_of_many_thin_rows(width, height):
     last = g.features(1, seed=3, camera=cam, crop=(width - crop_w, height - crop_h, crop_w, crop_h)).reshape(-1)
     assert torch.equal(out[:first.numel()], first)
     assert torch.equal(out[-last.numel():], last)
+
+
+@pytest.mark.parametrize("where", [200000, -1, (1 << 32) + 7])
+def test_texels_past_32_bits_are_checked(where):
+    """An environment of more than 2^32 floats with one negative texel is refused wherever it lies."""
+    from paper_2407_19977_gb300 import native as N
+    from paper_2407_19977_gb300.api import _ptr, _stream_handle
+    w, h = 65536, 21846
+    if torch.cuda.mem_get_info()[0] < 3 * w * h * 12:
+        pytest.skip("needs the environment's memory twice")
+    v = torch.tensor([[0, 0, 0], [1, 0, 0], [0, 1, 0]], dtype=torch.float32, device="cuda")
+    idx = torch.tensor([0, 1, 2], dtype=torch.int32, device="cuda")
+    mid = torch.zeros(1, dtype=torch.int32, device="cuda")
+    mats = (N.pt_openpbr * 1)()
+    from paper_2407_19977_gb300 import scenes
+    mats[0].v[:] = [float(x) for x in scenes.diffuse((.5, .5, .5))]
+    env = torch.zeros(w * h * 3, dtype=torch.float32, device="cuda")
+    env[where] = -1.0
+    out = C.c_void_p()
+    with pytest.raises(Exception):
+        N.call("pt_scene_create", _ptr(v), 3, _ptr(idx), 1, _ptr(mid), mats, 1, None, 0, _ptr(env), w, h, 1,
+               _stream_handle(), C.byref(out))
+    assert b"env texel" in N.load().pt_last_error()
