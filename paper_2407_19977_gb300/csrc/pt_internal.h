@@ -57,6 +57,7 @@ struct WaveBuffers {
     // (freed with the scene) instead of being freed
     bool recorded = false;
     std::vector<void*> retired;
+    bool small_auto = false;     // the large automatic wave did not fit: later calls don't try it
     void* block = nullptr;       // the allocation that holds the buffers up to `counters`
     float4* ray_o[2] = {nullptr, nullptr};   // queue entries: origin (w unused)
     float4* ray_d[2] = {nullptr, nullptr};   // direction, w = path id bits
@@ -188,7 +189,7 @@ pt_status pt_nrc_render_infer_dev(pt_nrc* N, const float* queries, const uint32_
                                   cudaStream_t st);
 uint32_t pt_nrc_frame_samples(const pt_nrc* N);
 uint64_t pt_nrc_serial(const pt_nrc* N);
-pt_status pt_nrc_render_prepare(pt_nrc* N, uint32_t infer_cap, uint32_t train_cap);
+pt_status pt_nrc_render_prepare(pt_nrc* N, uint32_t train_cap);
 // Series of the fuzz lobe (FUZZ_FLOATS per row) for n raw material rows of PT_OPENPBR_FLOATS
 // floats on the device; rows without fuzz get zeros (pt_fuzz.cu).
 pt_status pt_fuzz_series(const float* raw_materials, uint32_t n, float* out, cudaStream_t st);

@@ -1395,10 +1395,6 @@ struct pt_nrc {
     float *Y = nullptr, *dX = nullptr, *part = nullptr, *d_loss = nullptr;
     uint32_t* d_step = nullptr;   // Adam's step count (device)
     uint32_t* d_err = nullptr;     // device error word (1: a tensor-core wait ran out)
-    // inference buffers
-    uint32_t icap = 0;
-    __half* iX = nullptr;
-    float* iY = nullptr;
     float3 lo, inv_ext;
     uint64_t launches = 0;
 };
@@ -1518,8 +1514,7 @@ extern "C" void pt_nrc_destroy(pt_nrc* N) {
     if (!N) return;
     cudaDeviceSynchronize();
     void* ps[] = {N->d_res, N->d_w, N->d_wh, N->d_wm, N->d_wv, N->d_wg, N->d_grid, N->d_gh, N->d_gm, N->d_gv, N->d_gg,
-                  N->X, N->acts, N->dY, N->dZ, N->Y, N->dX, N->part, N->d_loss, N->iX, N->iY, N->d_err,
-                  N->d_step};
+                  N->X, N->acts, N->dY, N->dZ, N->Y, N->dX, N->part, N->d_loss, N->d_err, N->d_step};
     for (void* p : ps)
         if (p) cudaFree(p);
     delete N;
@@ -1530,7 +1525,8 @@ static uint32_t encode_grid(uint32_t cap, uint32_t L) {
     return (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>((threads + 255) / 256, 32ull * pt_num_sms()));
 }
 
-// forward (+ optional activations) of rc rows already resident on the device
+// forward of rc rows already resident on the device: with `acts` (training) the encoding goes to X
+// and the activations to acts, without (inference) neither is written
 static int g_infer_blocks = 0, g_infer_tc_blocks = 0;
 
 static pt_status nrc_forward(pt_nrc* N, const float* q, RowCount rc, __half* X, float* Y, __half* acts, cudaStream_t st) {
@@ -1673,14 +1669,8 @@ extern "C" pt_status pt_nrc_infer(pt_nrc* N, const float* queries, uint32_t n, f
     PT_CHECK_ARG(N && queries && out_rgb, "NULL argument");
     if (n == 0) return PT_OK;
     cudaStream_t st = (cudaStream_t)cuda_stream;
-    if (N->icap < n) {
-        if (N->iX) cudaFree(N->iX);
-        N->iX = nullptr;
-        PT_CUDA_TRY(cudaMalloc(&N->iX, (size_t)n * W * sizeof(__half)));
-        N->icap = n;
-    }
     // the MLP writes 4 floats per row; out_rgb is the caller's n x 4 buffer
-    return nrc_forward(N, queries, RowCount{n, nullptr, 0}, N->iX, out_rgb, nullptr, st);
+    return nrc_forward(N, queries, RowCount{n, nullptr, 0}, nullptr, out_rgb, nullptr, st);
 }
 
 extern "C" pt_status pt_nrc_params(pt_nrc* N, int which, float** ptr, uint64_t* count) {
@@ -1716,28 +1706,15 @@ extern "C" pt_status pt_nrc_last_loss(pt_nrc* N, float* loss) {
 }
 
 // ---- hooks used by the renderer: the row counts stay on the device (no host round trip) ----
-static pt_status ensure_infer(pt_nrc* N, uint32_t cap) {
-    if (N->icap >= cap) return PT_OK;
-    if (N->iX) cudaFree(N->iX);
-    N->iX = nullptr;
-    PT_CUDA_TRY(cudaMalloc(&N->iX, (size_t)cap * W * sizeof(__half)));
-    N->icap = cap;
-    return PT_OK;
-}
-
 // scratch for a renderer's calls, allocated before a graph capture (none happens inside one)
-pt_status pt_nrc_render_prepare(pt_nrc* N, uint32_t infer_cap, uint32_t train_cap) {
-    pt_status r = ensure_infer(N, infer_cap);
-    if (r != PT_OK) return r;
+pt_status pt_nrc_render_prepare(pt_nrc* N, uint32_t train_cap) {
     if (N->o.train_kernels == 0) return PT_OK;   // the fused training kernel needs no scratch
     return ensure_train(N, std::min(N->o.batch, std::max(train_cap, 1u)));
 }
 
 pt_status pt_nrc_render_infer_dev(pt_nrc* N, const float* queries, const uint32_t* n_dev, uint32_t cap, float* out4,
                                   cudaStream_t st) {
-    pt_status r = ensure_infer(N, cap);
-    if (r != PT_OK) return r;
-    return nrc_forward(N, queries, RowCount{cap, n_dev, 0}, N->iX, out4, nullptr, st);
+    return nrc_forward(N, queries, RowCount{cap, n_dev, 0}, nullptr, out4, nullptr, st);
 }
 
 uint32_t pt_nrc_frame_samples(const pt_nrc* N) { return N->o.frame_samples; }

@@ -1607,15 +1607,16 @@ static void drop_buffer(WaveBuffers& w, void* p) {
     else cudaFree(p);
 }
 
-// drops every buffer; what captures hold stays in `retired`
+// drops every buffer; what captures hold stays in `retired`, and whether the large wave fits is
+// remembered
 static void reset_wave(WaveBuffers& w) {
     void* ps[] = {w.block, w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id,
                   w.train_samples, w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
     for (void* p : ps) drop_buffer(w, p);
-    std::vector<void*> kept;
-    kept.swap(w.retired);
-    w = WaveBuffers();
-    w.retired.swap(kept);
+    WaveBuffers empty;
+    empty.retired.swap(w.retired);
+    empty.small_auto = w.small_auto;
+    w = std::move(empty);
 }
 
 pt_status pt_free_wave(WaveBuffers& w) {
@@ -1644,16 +1645,20 @@ static void carve_wave(WaveBuffers& w, void* block, size_t c) {
     w.bytes = wave_bytes(c);
 }
 
-// one allocation for all of a wave's buffers (13 of them took 0.45 ms of a scene's first frame)
-static pt_status ensure_wave(WaveBuffers& w, uint32_t capacity) {
+// one allocation for all of a wave's buffers (13 of them took 0.45 ms of a scene's first frame);
+// with `try_only` the present buffers stay as they are if there is no room for the new ones
+// beside them
+static pt_status ensure_wave(WaveBuffers& w, uint32_t capacity, bool try_only = false) {
     if (w.capacity >= capacity) return PT_OK;
-    reset_wave(w);
+    if (!try_only) reset_wave(w);
     void* block = nullptr;
     const cudaError_t e = cudaMalloc(&block, wave_bytes(capacity));
     if (e != cudaSuccess) {
+        cudaGetLastError();     // not for the next call to find
         pt_set_error(std::string("wavefront buffers: ") + cudaGetErrorString(e));
         return PT_ERR_OOM;
     }
+    if (try_only) reset_wave(w);
     carve_wave(w, block, capacity);
     w.block = block;
     return PT_OK;
@@ -1666,6 +1671,9 @@ static pt_status ensure_nrc_buffers(WaveBuffers& w, uint32_t rec_per_path, uint3
     if (w.nrc_capacity >= cap && w.rec_per_path >= rec_per_path && w.sample_cap == samples) return PT_OK;
     void* ps[] = {w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id, w.train_samples};
     for (void* q : ps) drop_buffer(w, q);
+    w.aux = w.nrc_counters = w.train_nv = w.train_id = nullptr;
+    w.nrc_q = w.nrc_out = w.train_rec = w.train_samples = nullptr;
+    w.nrc_capacity = 0;
     PT_CUDA_TRY(cudaMalloc(&w.aux, (size_t)cap * sizeof(uint32_t)));
     PT_CUDA_TRY(cudaMalloc(&w.nrc_q, (size_t)cap * 16 * sizeof(float)));
     PT_CUDA_TRY(cudaMalloc(&w.nrc_out, (size_t)cap * 4 * sizeof(float)));
@@ -1758,15 +1766,16 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                                   pt_accum* acc, const pt_render_opts& o, cudaStream_t user_st) {
     cudaStream_t st = user_st;   // the stream the wave loops below issue to (a capture stream while capturing)
     const uint32_t npix_total = acc->width * acc->height;
-    // automatic wave: 2^23 paths (1.4 GB of queues), or 2^21 where there is no room for that, in
-    // frames that train the cache (a wave is a training set) and under stream capture, where the
-    // buffers of an earlier, smaller call cannot grow.  Every pass of a wave ends with
+    // automatic wave: 2^23 paths (1.4 GB of queues), or 2^21 where there is no room for that (with
+    // the reservoir or cache buffers of its paths), in frames that train the cache (a wave is a
+    // training set) and under stream capture, where the buffers of an earlier, smaller call
+    // cannot grow.  Every pass of a wave ends with
     // the chip waiting for its longest rays, so few large waves beat many small ones: 2^21 /
     // 2^22 / 2^23 / 2^24 paths a wave, 512 x 512 still of 25 samples 10.12 / 7.93 / 6.84 / 6.84
     // ms, glass scene at 1917 x 1079 and 2 samples 5.85 / 4.20 / 4.21 / 4.23.
     constexpr uint32_t LARGE_WAVE = 1u << 23, SMALL_WAVE = 1u << 21;
     const bool captured = capturing(user_st);
-    const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train) && !captured;
+    const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train) && !captured && !s->wave.small_auto;
     uint32_t cap = std::max(o.wave_paths ? o.wave_paths : large ? LARGE_WAVE : SMALL_WAVE, 32u);
     // waves hold whole samples of a pixel range: pixel chunk <= cap, then samples per wave;
     // with ReSTIR the chunk is the whole window (the spatial pass reads any pixel of it)
@@ -1774,18 +1783,25 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
     const bool coop = o.traversal == PT_TRAVERSAL_COOP;
     WaveBuffers& w = s->wave;
     uint32_t pix_chunk = 0, samp_per_wave = 0;
-    auto buffers = [&]() -> pt_status {
+    auto buffers = [&](bool try_only) -> pt_status {
         pix_chunk = restir ? npix_total : std::min(npix_total, cap);
         samp_per_wave = std::max(1u, std::min(spp, cap / pix_chunk));
-        const pt_status e = ensure_wave(w, pix_chunk * samp_per_wave);
-        return e == PT_OK && restir ? ensure_restir_buffers(w) : e;
+        pt_status e = ensure_wave(w, pix_chunk * samp_per_wave, try_only);
+        if (e == PT_OK && restir) e = ensure_restir_buffers(w);
+        if (e == PT_OK && o.nrc) e = ensure_nrc_buffers(w, std::min(max_depth + 1, 16u), pt_nrc_frame_samples(o.nrc));
+        return e;
     };
-    pt_status r = buffers();
-    if (r == PT_ERR_OOM && large) {
-        cudaGetLastError();
-        reset_wave(w);
-        cap = SMALL_WAVE;
-        r = buffers();
+    pt_status r = buffers(large || captured);
+    if (r == PT_ERR_OOM && !captured) {
+        // queues that were in place, or fitted, without room for what goes with them are given up
+        const bool queues = w.capacity >= pix_chunk * samp_per_wave;
+        if (large || queues) {
+            cudaGetLastError();
+            if (queues) reset_wave(w);
+            if (large) cap = SMALL_WAVE;
+            w.small_auto = w.small_auto || large;
+            r = buffers(false);
+        }
     }
     if (r != PT_OK) return r;
     // from here on a caller's graph may hold the buffers' addresses
@@ -1830,9 +1846,7 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
         P.rs_g0 = w.rs_g0; P.rs_g1 = w.rs_g1; P.rs_gn = w.rs_gn; P.rs_i = w.rs_i; P.rs_f = w.rs_f;
     }
     if (o.nrc) {
-        r = ensure_nrc_buffers(w, std::min(max_depth + 1, 16u), pt_nrc_frame_samples(o.nrc));
-        if (r != PT_OK) return r;
-        r = pt_nrc_render_prepare(o.nrc, pix_chunk * samp_per_wave, w.sample_cap);
+        r = pt_nrc_render_prepare(o.nrc, w.sample_cap);
         if (r != PT_OK) return r;
         P.nrc_on = 1;
         P.rec_per_path = w.rec_per_path;
