@@ -2104,7 +2104,8 @@ static uint32_t auto_mode(const pt_render_opts& o, uint32_t npix, uint32_t spp, 
                                o.traversal || o.sort_by_material >= 0 || (o.flags & FLAG_COUNT);
         return few && !wave_opts ? PT_MODE_MEGAKERNEL : PT_MODE_WAVEFRONT;
     }
-    if (few) return PT_MODE_MEGAKERNEL;
+    // a small frame's waves limited to as few paths: as many launch sequences of the wavefront
+    if (few || (o.wave_paths && o.wave_paths < AUTO_WAVE_PATHS)) return PT_MODE_MEGAKERNEL;
     // a small frame that is being captured allocates nothing: the path kernel needs no buffers
     return capturing(st) ? PT_MODE_MEGAKERNEL : PT_MODE_WAVEFRONT;
 }
