@@ -616,18 +616,13 @@ __device__ __forceinline__ uint32_t byte_of(uint32_t lo4, uint32_t hi4, int i) {
 struct TravRay {
     float3 o, inv;
 };
-__device__ __forceinline__ float rcp_approx(float x) {   // within 1 ulp
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
 __device__ __forceinline__ TravRay make_trav(float3 o, float3 d) {
     TravRay r;
     r.o = o;
     const float big = 1e20f;
-    r.inv = mk3(fabsf(d.x) > 1e-20f ? rcp_approx(d.x) : copysignf(big, d.x),
-                fabsf(d.y) > 1e-20f ? rcp_approx(d.y) : copysignf(big, d.y),
-                fabsf(d.z) > 1e-20f ? rcp_approx(d.z) : copysignf(big, d.z));
+    r.inv = mk3(fabsf(d.x) > 1e-20f ? 1.0f / d.x : copysignf(big, d.x),
+                fabsf(d.y) > 1e-20f ? 1.0f / d.y : copysignf(big, d.y),
+                fabsf(d.z) > 1e-20f ? 1.0f / d.z : copysignf(big, d.z));
     return r;
 }
 
@@ -661,10 +656,10 @@ __device__ __forceinline__ NodeView load_node(const uint4* __restrict__ nodes, u
 // b = scale/d.  The byte q is read as the float f = 2^15 + q (the byte placed in the mantissa
 // of 2^15, no conversion instruction), and the distance is fma(f, b, c) with
 // c = a - 2^15 b.  e widens every slab by a bound on the rounding of those terms, in units of
-// u = 2^-24: the reciprocal, subtraction and product in a (4 u |a|), b (3 u over at most
+// u = 2^-24: the reciprocal, subtraction and product in a (3 u |a|), b (2 u over at most
 // 255 |b|), the builder's one-rounding decode of the plane (u |plane/d| <= u (|a| + |o/d| +
 // 255 |b|)), the fma's result (u (|a| + 255 |b|)), c and c -+ e (2 u (|a| + 2^15 |b|)): at
-// most 4.8e-7 |a| + 4.1e-3 |b| + 6e-8 |o/d|, so the test stays conservative.  The term in b is
+// most 4.2e-7 |a| + 4e-3 |b| + 6e-8 |o/d|, so the test stays conservative.  The term in b is
 // taken from c, |b| <= 2^-15 (|c| + |a|): where 2^15 b overflows, c and with it e are infinite,
 // so that c - e is -inf or NaN and c + e is +inf or NaN, as they are for a or b infinite.  Either
 // way the minimum and maximum ignore that axis and the box is tested on the others only, which
