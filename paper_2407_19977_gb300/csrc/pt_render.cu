@@ -215,8 +215,10 @@ static pt_status launch_megakernel_one(const DJob& job, uint32_t block_size, boo
                                        uint64_t* launches) {
     const uint32_t npix = job.cw * job.ch;
     const uint32_t threads = block_size ? std::min(std::max(32u, block_size & ~31u), PATH_THREADS) : PATH_THREADS;
-    const uint32_t S = std::min(job.spp, 32u), pix = threads / S;
-    const uint32_t grid = (npix + pix - 1) / pix;
+    // fewer samples side by side where a frame of 2^31 pixels would have more blocks than a grid
+    uint32_t S = std::min(job.spp, 32u);
+    while (((uint64_t)npix + threads / S - 1) / (threads / S) > 0x7fffffffu) S = (S + 1) / 2;
+    const uint32_t pix = threads / S, grid = (uint32_t)(((uint64_t)npix + pix - 1) / pix);
     if (fuzz) PT_LAUNCH(k_megakernel_one<true>, grid, threads, 0, st, job, S, pix);
     else PT_LAUNCH(k_megakernel_one<false>, grid, threads, 0, st, job, S, pix);
     (*launches)++;
