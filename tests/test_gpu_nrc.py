@@ -372,3 +372,25 @@ def test_nrc_gain_on_enclosed_scene():
     cached = g.render(4, seed=5, mode=1, nrc=net)
     e_plain, e_nrc = relmse(plain.image()), relmse(cached.image())
     assert e_nrc < 0.8 * e_plain, (e_nrc, e_plain)
+
+
+@pytest.mark.parametrize("batch,samples", [(8192, 32768), (4096, 9001)])
+def test_nrc_trainings_differ_by_no_more_than_their_summation_order(batch, samples):
+    """Two trainings from the same parameters and records.  The grid's gradients are FP32 atomic
+    sums in no fixed order: a step touches at most 128 entries (256 values) a sample, and a value
+    whose contributions cancel to within their rounding (some 10 x 2^-24 of their sum of sizes, so
+    about one in a million) may take either sign, which Adam's first steps turn into +-lr.  A few
+    such values a step, and the values of the samples that read them, may move by lr; nothing
+    else may: at most 1 value in 500 by more than lr / 100, 3 % of the table's norm, 1e-3 of the
+    weights'."""
+    from paper_2407_19977_gb300 import api
+    rec = torch.from_numpy(_records(np.random.default_rng(6), samples)).cuda()
+    out = []
+    for _ in range(3):
+        net = api.Nrc(seed=3, batch=batch, box=((0.0, 0.0, 0.0), (1.0, 1.0, 1.0)))
+        net.train(rec)
+        out.append((net.params(0).double().clone(), net.params(1).double().clone()))
+    for w, g in out[1:]:
+        assert float((w - out[0][0]).norm() / out[0][0].norm()) <= 1e-3
+        assert float((g - out[0][1]).norm() / out[0][1].norm()) <= 3e-2
+        assert float(((g - out[0][1]).abs() > 1e-4).double().mean()) <= 2e-3
