@@ -193,9 +193,10 @@ typedef struct {
     uint32_t mode;              /* PT_MODE_* */
     uint32_t wave_paths;        /* wavefront: paths per wave (0 = automatic: 2^23, or 2^21 when the
                                    cache is trained, under stream capture, and in a scene where
-                                   the larger wave's buffers once did not fit).  A wave of 2^23
-                                   paths holds 1.4 GB, one of 2^21 0.35 GB, kept by the scene until
-                                   it is destroyed; a call of fewer paths holds those of its paths */
+                                   the larger wave's buffers once would have taken more than a
+                                   sixteenth of the free device memory).  A wave of 2^23 paths
+                                   holds 1.4 GB, one of 2^21 0.35 GB, kept by the scene until it is
+                                   destroyed; a call of fewer paths holds those of its paths */
     int32_t sort_by_material;   /* wavefront: -1 automatic, 0 off, 1 on */
     uint32_t block_size;        /* threads per block (0 = automatic) */
     float* sample_out;          /* optional DEVICE buffer, height*width*spp*3 floats: the

@@ -1648,19 +1648,25 @@ static void carve_wave(WaveBuffers& w, void* block, size_t c) {
 }
 
 // one allocation for all of a wave's buffers (13 of them took 0.45 ms of a scene's first frame);
-// with `try_only` the present buffers stay as they are if there is no room for the new ones
-// beside them
-static pt_status ensure_wave(WaveBuffers& w, uint32_t capacity, bool try_only = false) {
+// with `keep` the present buffers stay as they are if there is no room for the new ones beside
+// them, with `roomy` there is room if they take at most a sixteenth of the free memory
+static pt_status ensure_wave(WaveBuffers& w, uint32_t capacity, bool keep = false, bool roomy = false) {
     if (w.capacity >= capacity) return PT_OK;
-    if (!try_only) reset_wave(w);
     void* block = nullptr;
-    const cudaError_t e = cudaMalloc(&block, wave_bytes(capacity));
+    cudaError_t e = cudaSuccess;
+    if (roomy) {
+        size_t free_bytes = 0, total_bytes = 0;
+        e = cudaMemGetInfo(&free_bytes, &total_bytes);
+        if (e == cudaSuccess && wave_bytes(capacity) > free_bytes / 16) e = cudaErrorMemoryAllocation;
+    }
+    if (!keep) reset_wave(w);
+    if (e == cudaSuccess) e = cudaMalloc(&block, wave_bytes(capacity));
     if (e != cudaSuccess) {
         cudaGetLastError();     // not for the next call to find
         pt_set_error(std::string("wavefront buffers: ") + cudaGetErrorString(e));
         return PT_ERR_OOM;
     }
-    if (try_only) reset_wave(w);
+    if (keep) reset_wave(w);
     carve_wave(w, block, capacity);
     w.block = block;
     return PT_OK;
@@ -1768,13 +1774,14 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
                                   pt_accum* acc, const pt_render_opts& o, cudaStream_t user_st) {
     cudaStream_t st = user_st;   // the stream the wave loops below issue to (a capture stream while capturing)
     const uint32_t npix_total = acc->width * acc->height;
-    // automatic wave: 2^23 paths (1.4 GB of queues), or 2^21 where there is no room for that (with
-    // the reservoir or cache buffers of its paths), in frames that train the cache (a wave is a
+    // automatic wave: 2^23 paths (1.4 GB of queues), or 2^21 (0.35 GB) where the larger one would
+    // take more than a sixteenth of the free memory (each scene keeps its own, and many scenes
+    // may be open) or what goes with it does not fit, in frames that train the cache (a wave is a
     // training set) and under stream capture, where the buffers of an earlier, smaller call
-    // cannot grow.  Every pass of a wave ends with
-    // the chip waiting for its longest rays, so few large waves beat many small ones: 2^21 /
-    // 2^22 / 2^23 / 2^24 paths a wave, 512 x 512 still of 25 samples 10.12 / 7.93 / 6.84 / 6.84
-    // ms, glass scene at 1917 x 1079 and 2 samples 5.85 / 4.20 / 4.21 / 4.23.
+    // cannot grow.  Every pass of a wave ends with the chip waiting for its longest rays, so few
+    // large waves beat many small ones: 2^21 / 2^22 / 2^23 / 2^24 paths a wave, 512 x 512 still of
+    // 25 samples 10.12 / 7.93 / 6.84 / 6.84 ms, glass scene at 1917 x 1079 and 2 samples 5.85 /
+    // 4.20 / 4.21 / 4.23.
     constexpr uint32_t LARGE_WAVE = 1u << 23, SMALL_WAVE = 1u << 21;
     const bool captured = capturing(user_st);
     const bool large = o.wave_paths == 0 && !(o.nrc && o.nrc_train) && !captured && !s->wave.small_auto;
@@ -1785,24 +1792,25 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
     const bool coop = o.traversal == PT_TRAVERSAL_COOP;
     WaveBuffers& w = s->wave;
     uint32_t pix_chunk = 0, samp_per_wave = 0;
-    auto buffers = [&](bool try_only) -> pt_status {
+    auto buffers = [&](bool roomy) -> pt_status {
         pix_chunk = restir ? npix_total : std::min(npix_total, cap);
         samp_per_wave = std::max(1u, std::min(spp, cap / pix_chunk));
-        pt_status e = ensure_wave(w, pix_chunk * samp_per_wave, try_only);
+        pt_status e = ensure_wave(w, pix_chunk * samp_per_wave, roomy || captured, roomy);
         if (e == PT_OK && restir) e = ensure_restir_buffers(w);
         if (e == PT_OK && o.nrc) e = ensure_nrc_buffers(w, std::min(max_depth + 1, 16u), pt_nrc_frame_samples(o.nrc));
         return e;
     };
-    pt_status r = buffers(large || captured);
+    pt_status r = buffers(large);
     if (r == PT_ERR_OOM && !captured) {
         // queues that were in place, or fitted, without room for what goes with them are given up
-        const bool queues = w.capacity >= pix_chunk * samp_per_wave;
+        const uint32_t tried = pix_chunk * samp_per_wave;
+        const bool queues = w.capacity >= tried;
         if (large || queues) {
             cudaGetLastError();
             if (queues) reset_wave(w);
             if (large) cap = SMALL_WAVE;
-            w.small_auto = w.small_auto || large;
             r = buffers(false);
+            w.small_auto = w.small_auto || pix_chunk * samp_per_wave < tried;
         }
     }
     if (r != PT_OK) return r;

@@ -103,6 +103,23 @@ def test_smaller_waves_where_the_large_one_does_not_fit(kind, spp, leave):
         assert g.stats()["graph_replays"] == 2
 
 
+@pytest.mark.parametrize("leave,most", [(15, 360 << 20), (17, 1200 << 20)])
+def test_large_wave_takes_a_sixteenth_of_the_free_memory_at_most(leave, most):
+    """3 samples of 2.15M pixels: 1.08 GB of queues in one wave, 0.36 in waves of one sample."""
+    from paper_2407_19977_gb300 import api, native as N, scenes
+    w, h = 1536, 1400
+    sc = scenes.cornell_box(seed=2, width=w, height=h, max_depth=3)
+    want = api.Scene(sc).render(3, seed=5, mode=N.PT_MODE_MEGAKERNEL)
+    g = api.Scene(sc)
+    acc = api.Accum(w, h)
+    with _only(leave * 3 * w * h * 168 + (16 << 20)):
+        before = _used()
+        g.render(3, seed=5, accum=acc)
+        grown = _used() - before
+    assert most * 0.85 < grown <= most
+    assert torch.equal(acc.sum, want.sum) and torch.equal(acc.comp, want.comp)
+
+
 def test_small_frame_without_room_for_a_wave():
     """A small frame that AUTO sends to the wavefront renders all the same where no wave fits."""
     from paper_2407_19977_gb300 import api, native as N, scenes
