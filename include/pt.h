@@ -249,7 +249,7 @@ enum {
  *               codes' highest differing bit whatever the triangles' sizes);
  *  PT_BVH_PLOC  parallel locally-ordered clustering (Meister & Bittner 2018): rounds in which
  *               each cluster merges with its mutual nearest neighbour by surface area within
- *               16 positions in the Morton order (a tree close to a full SAH build; the
+ *               8 positions in the Morton order (a tree close to a full SAH build; the
  *               default). */
 enum { PT_BVH_DEFAULT = 0, PT_BVH_LBVH = 1, PT_BVH_PLOC = 2 };
 

@@ -328,9 +328,11 @@ __global__ void k_bottom_up(BinTree T, int n, const uint32_t* par_int, const uin
 // node's children have higher indices than the node.  A top-down pass over the rounds in
 // reverse then lays the triangles out in tree order, giving each subtree the contiguous
 // [first, last] range the collapse needs.
-// 8, 16 and 32 give equally good trees (closest-hit passes of the 1080p CAD frame 2.99 / 3.03 /
-// 2.99 ms, of the glass scene 2.11 / 2.18 / 2.18) and the search grows with it: opening a
-// 1.07M-triangle model takes 5.1 / 5.5 / 5.95 ms.
+// 8 against the published 16: builds take 6 % less (0.2M-triangle CAD model 2.02 -> 1.79 ms,
+// 5.2M-triangle glass scene 5.9 -> 5.5).  Frames of 22 CAD, glass and velvet scenes of 640 to 5.2M
+// triangles differ by -1.7 to +2.2 % (mean 0.1 %; fewer node visits in 12, more in 10), as after
+// any small change of the tree.  A random soup, whose Morton order says little about its sizes,
+// is the exception: 2.8 % (20,000 triangles) and 6.5 % (300,000) longer frames.
 constexpr int PLOC_R = 8;
 constexpr int PLOC_THREADS = 256;
 constexpr int PLOC_SCAN_ITEMS = 4;                      // per thread of the block scan

@@ -775,11 +775,10 @@ __device__ __forceinline__ void closest_init(const DScene& S, float3 o, float3 d
 // the PT_STACK entries the traversal may use is checked once after it.
 // BRANCHLESS selects the form of the child loop; both push the same children in the same
 // order.  The branching form (a slot that misses skips the push logic) suits coherent rays: the
-// feature pass takes it (1080p preview 3.34 -> 3.28 ms; the per-bounce passes, which took it
-// before they went in stages, 3.99 -> 3.68).  The out-of-line traversal that the tail kernel and the megakernel call takes the form without
-// branches, which measured faster there (tail kernel 0.49 -> 0.41 ms a step on the same
-// frame, 1.45 -> 1.19 ms on the 5.2M-triangle scene), where the lanes of a warp are at
-// different bounces and stages.
+// feature pass takes it (1080p preview 3.34 -> 3.28 ms).  The out-of-line traversal of the path
+// kernel and the batch megakernel takes the form without branches, which suits warps whose lanes
+// are at different bounces (in the tail kernel, before it had loops of its own, 0.49 -> 0.41 ms a
+// 1080p CAD step).
 #define PT_STACK_SLACK 7
 template <bool COUNT, bool BRANCHLESS = false>
 __device__ __forceinline__ bool closest_step(const DScene& S, ClosestState& st, uint2 (&stack)[PT_STACK + PT_STACK_SLACK],
@@ -1342,9 +1341,10 @@ static __device__ __noinline__ bool trace_any(const DScene& S, float3 o, float3 
 
 // The same for the tail kernel, whose paths are at different vertices: the node visits of the
 // staged passes (loops over the children that are hit, where the loops above have a body per
-// slot).  Same visits in the same order.  Glass scene's tail 0.91 -> 0.86 ms (the frame 3.65 ->
-// 3.51), 1080p preview with features and denoiser 3.03 -> 3.00; but a 64 x 64 Cornell frame in
-// the path kernel, where a warp's rays are alike, 0.20 -> 0.23, so that keeps the loops above.
+// slot).  Same visits in the same order.  Against the loops above, medians of five processes in
+// turn, which differ by 0.2 % among themselves: glass scene's frame 3.87 -> 3.84 ms, velvet 2.61 ->
+// 2.59, 1080p preview with features and denoiser 3.34 -> 3.31; but a 64 x 64 Cornell frame in the
+// path kernel, where a warp's rays are alike, 0.20 -> 0.23, so that keeps the loops above.
 static __device__ __noinline__ void tail_closest(const DScene& S, float3 o, float3 d, float tmax, HitRec& h) {
     LaneRay r;
     uint2 stack[PT_STACK + PT_STACK_SLACK];

@@ -61,7 +61,7 @@ struct WaveBuffers {
     void* block = nullptr;       // the allocation that holds the buffers up to `counters`
     float4* ray_o[2] = {nullptr, nullptr};   // queue entries: origin (w unused)
     float4* ray_d[2] = {nullptr, nullptr};   // direction, w = path id bits
-    float4* hit = nullptr;       // t, u, v, tri bits (per queue slot)
+    float4* hit = nullptr;       // per queue slot: t and, in w, the triangle (y and z unused)
     float4* beta = nullptr;      // per path: beta.xyz, prev_pdf
     float4* radiance = nullptr;  // per path: L.xyz
     float4* sh_o = nullptr;      // shadow queue: origin, tmax

@@ -282,9 +282,11 @@ __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const __half* p) {
 // a shared-memory tile (never written to HBM).  Lanes 2l and 2l + 1 encode level l of queries
 // 2r and 2r + 1 (r = 0..7): each gathers one x side of both queries' cells, so the two corners
 // along x, which lie in one 32-byte sector 7 times in 8, are one access of the pair, and the
-// values are exchanged and summed in corner order.  Bound by the L2 sectors of the fine levels
-// (1,000,003 random queries: 437 us with a whole cell per lane, 426 in pairs).  The tile then
-// feeds the same tensor-core layers as k_mlp_forward, with the A fragments read by ldmatrix.
+// values are exchanged and summed in corner order (1,000,003 random queries: 437 us with a whole
+// cell per lane, 426 in pairs).  No unit is at its rate: 60 % of the issue slots, L1 59 % (a
+// gather touches 8 sectors, 82 a query in all), L2 45 %, tensor pipe 14 %; what is left is the
+// gathers' latency (long-scoreboard stalls 3.6 per issue) with half the warp slots filled.  The
+// tile then feeds the same tensor-core layers as k_mlp_forward, with the A fragments read by ldmatrix.
 // 512 threads share one copy of the weights in shared memory (the copy, not the registers,
 // limited 128-thread blocks to 4 per SM); two blocks of sixteen warps fit per SM (64
 // registers, no spills)

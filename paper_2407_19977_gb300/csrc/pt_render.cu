@@ -658,7 +658,8 @@ __device__ __forceinline__ uint32_t hit_key(const DScene& S, const HitRec& h, ui
 // triangles as soon as a third of the live lanes wait for one, else nodes.  Once TRACE_REFILL
 // lanes have finished, the warp writes their hits and takes as many new rays with one atomic,
 // so the latency of those loads and stores is paid for 20 lanes at a time.
-// Bound by issue slots and the ALU pipe (71 % and 64 % busy; the tree stays in L2).  Measured
+// Bound by issue slots and the ALU pipe (68-75 % and 63-66 % busy in the launches of the first two
+// bounces; the tree stays in L2).  Measured
 // on the 1080p CAD frame, 8.3M paths (closest-hit passes of one step): one ray per lane until
 // all 32 of the warp are done, divergence left to the hardware, 3.58 ms at 10 active lanes
 // per instruction; in stages 2.97 ms at 17 active lanes.  Refill at 8 / 12 / 16 / 20 / 24 / 32
@@ -2260,8 +2261,8 @@ static pt_status batch_wavefront(const pt_job* jobs, uint32_t n_jobs, uint32_t K
 // A wave is a list of segments (WfmSeg), filled in job order: each job's (pixel range x
 // sample range) blocks are the ones a single-scene wavefront of that job would make, and a
 // block that does not fit in the wave's remaining room is split along its pixels.  Every
-// wave runs the single-scene launch sequence (raygen, per bounce: setup, tail, closest hit,
-// shade, shadow rays; accumulation) once for all its jobs, the kernels looking each path's
+// wave runs the single-scene launch sequence (raygen, per bounce: rays, tail, sort, shade;
+// accumulation) once for all its jobs, the kernels looking each path's
 // scene, camera, depth and seed up through its segment.  The launch sequence of a batch
 // layout is captured once as a CUDA graph (with the job table copied in from pinned memory
 // at its start, so seeds, first samples and cameras may change between calls) and replayed.
