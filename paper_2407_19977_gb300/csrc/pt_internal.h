@@ -52,10 +52,10 @@ enum { ST_EXT = 0, ST_SHADOW = 1, ST_PATHS = 2, ST_NAN = 3, ST_RR = 4, ST_NRC = 
 // ---- wavefront workspace ---------------------------------------------------------------
 struct WaveBuffers {
     uint32_t capacity = 0;       // paths per wave
-    // a caller's stream capture has recorded addresses of these buffers: its graph may be
-    // replayed as long as the scene lives, so buffers that are replaced then go to `retired`
-    // (freed with the scene) instead of being freed
-    bool recorded = false;
+    // a caller's stream capture has recorded addresses of the block, the cache's or the
+    // reservoirs' buffers: its graph may be replayed as long as the scene lives, so those that are
+    // replaced then go to `retired` (freed with the scene) instead of being freed
+    bool block_recorded = false, nrc_recorded = false, restir_recorded = false;
     std::vector<void*> retired;
     bool small_auto = false;     // the large automatic wave did not fit: later calls don't try it
     void* block = nullptr;       // the allocation that holds the buffers up to `counters`

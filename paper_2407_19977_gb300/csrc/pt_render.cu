@@ -1604,18 +1604,33 @@ __global__ void k_wf_accum(WfParams P) {
 }
 
 // a buffer that is replaced: freed, or kept for the graphs that may hold its address
-static void drop_buffer(WaveBuffers& w, void* p) {
+static void drop_buffer(WaveBuffers& w, void* p, bool recorded) {
     if (!p) return;
-    if (w.recorded) w.retired.push_back(p);
+    if (recorded) w.retired.push_back(p);
     else cudaFree(p);
+}
+static void drop_nrc_buffers(WaveBuffers& w) {
+    void* ps[] = {w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id, w.train_samples};
+    for (void* p : ps) drop_buffer(w, p, w.nrc_recorded);
+    w.aux = w.nrc_counters = w.train_nv = w.train_id = nullptr;
+    w.nrc_q = w.nrc_out = w.train_rec = w.train_samples = nullptr;
+    w.nrc_capacity = 0;
+    w.nrc_recorded = false;
+}
+static void drop_restir_buffers(WaveBuffers& w) {
+    void* ps[] = {w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
+    for (void* p : ps) drop_buffer(w, p, w.restir_recorded);
+    w.rs_g0 = w.rs_g1 = w.rs_gn = w.rs_i = w.rs_f = nullptr;
+    w.restir_capacity = 0;
+    w.restir_recorded = false;
 }
 
 // drops every buffer; what captures hold stays in `retired`, and whether the large wave fits is
 // remembered
 static void reset_wave(WaveBuffers& w) {
-    void* ps[] = {w.block, w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id,
-                  w.train_samples, w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
-    for (void* p : ps) drop_buffer(w, p);
+    drop_buffer(w, w.block, w.block_recorded);
+    drop_nrc_buffers(w);
+    drop_restir_buffers(w);
     WaveBuffers empty;
     empty.retired.swap(w.retired);
     empty.small_auto = w.small_auto;
@@ -1678,11 +1693,7 @@ static pt_status ensure_wave(WaveBuffers& w, uint32_t capacity, bool keep = fals
 static pt_status ensure_nrc_buffers(WaveBuffers& w, uint32_t rec_per_path, uint32_t samples) {
     const uint32_t cap = w.capacity, slots = std::max(samples / 2, 1u);
     if (w.nrc_capacity >= cap && w.rec_per_path >= rec_per_path && w.sample_cap == samples) return PT_OK;
-    void* ps[] = {w.aux, w.nrc_q, w.nrc_out, w.nrc_counters, w.train_rec, w.train_nv, w.train_id, w.train_samples};
-    for (void* q : ps) drop_buffer(w, q);
-    w.aux = w.nrc_counters = w.train_nv = w.train_id = nullptr;
-    w.nrc_q = w.nrc_out = w.train_rec = w.train_samples = nullptr;
-    w.nrc_capacity = 0;
+    drop_nrc_buffers(w);
     PT_CUDA_TRY(cudaMalloc(&w.aux, (size_t)cap * sizeof(uint32_t)));
     PT_CUDA_TRY(cudaMalloc(&w.nrc_q, (size_t)cap * 16 * sizeof(float)));
     PT_CUDA_TRY(cudaMalloc(&w.nrc_out, (size_t)cap * 4 * sizeof(float)));
@@ -1701,10 +1712,7 @@ static pt_status ensure_nrc_buffers(WaveBuffers& w, uint32_t rec_per_path, uint3
 // ReSTIR DI buffers for every path of a wave
 static pt_status ensure_restir_buffers(WaveBuffers& w) {
     if (w.restir_capacity >= w.capacity) return PT_OK;
-    void* ps[] = {w.rs_g0, w.rs_g1, w.rs_gn, w.rs_i, w.rs_f};
-    for (void* q : ps) drop_buffer(w, q);
-    w.rs_g0 = w.rs_g1 = w.rs_gn = w.rs_i = w.rs_f = nullptr;
-    w.restir_capacity = 0;
+    drop_restir_buffers(w);
     const size_t c = w.capacity;
     PT_CUDA_TRY(cudaMalloc(&w.rs_g0, c * sizeof(float4)));
     PT_CUDA_TRY(cudaMalloc(&w.rs_g1, c * sizeof(float4)));
@@ -1797,6 +1805,12 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
         pix_chunk = restir ? npix_total : std::min(npix_total, cap);
         samp_per_wave = std::max(1u, std::min(spp, cap / pix_chunk));
         pt_status e = ensure_wave(w, pix_chunk * samp_per_wave, roomy || captured, roomy);
+        if (captured && e == PT_OK) {
+            // from here on a caller's graph may hold the addresses (and nothing is freed in a capture)
+            w.block_recorded = true;
+            w.nrc_recorded = w.nrc_recorded || o.nrc;
+            w.restir_recorded = w.restir_recorded || restir;
+        }
         if (e == PT_OK && restir) e = ensure_restir_buffers(w);
         if (e == PT_OK && o.nrc) e = ensure_nrc_buffers(w, std::min(max_depth + 1, 16u), pt_nrc_frame_samples(o.nrc));
         return e;
@@ -1815,8 +1829,10 @@ static pt_status render_wavefront(pt_scene* s, const pt_camera& cam, uint32_t sp
         }
     }
     if (r != PT_OK) return r;
-    // from here on a caller's graph may hold the buffers' addresses
-    w.recorded = w.recorded || captured;
+    if (captured) {
+        w.nrc_recorded = w.nrc_recorded || o.nrc;            // a set allocated just now, too
+        w.restir_recorded = w.restir_recorded || restir;
+    }
     const bool sort = o.sort_by_material == 1 || (o.sort_by_material < 0 && s->n_mats + 2 <= MAX_SORT_KEYS && s->n_mats > 1);
     const uint32_t n_keys = (sort && s->n_mats + 2 <= MAX_SORT_KEYS) ? s->n_mats + 2 : 0;
     wf_occupancy();

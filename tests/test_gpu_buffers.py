@@ -131,3 +131,29 @@ def test_small_frame_without_room_for_a_wave():
             acc.reset()
             g.render(64, seed=5, accum=acc)
             assert torch.equal(acc.sum, want.sum) and torch.equal(acc.comp, want.comp)
+
+
+def test_only_recorded_buffers_are_kept():
+    """After a capture, calls that replace the cache's buffers again and again (two caches of
+    different training sets) keep the recorded set and no other; the captured graph replays."""
+    from paper_2407_19977_gb300 import api, native as N, scenes
+    w, h = 1024, 640
+    sc = scenes.cornell_box(seed=2, width=w, height=h, max_depth=3)
+    lo, hi = tuple(sc.vertices.min(0) - 0.01), tuple(sc.vertices.max(0) + 0.01)
+    g = api.Scene(sc)
+    nets = [api.Nrc(seed=3, box=(lo, hi), frame_samples=1 << k) for k in (15, 16)]
+    acc, other = api.Accum(w, h), api.Accum(w, h)
+    opts = dict(seed=5, mode=N.PT_MODE_WAVEFRONT)
+    want = g.render(1, nrc=nets[0], **opts)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        g.render(1, nrc=nets[0], accum=acc, **opts)
+    used = []
+    for k in range(6):
+        g.render(1, nrc=nets[k % 2], accum=other, **opts)
+        g.render(1, nrc=nets[(k + 1) % 2], accum=other, **opts)
+        used.append(_used())
+    assert used[-1] == used[1]
+    acc.reset()
+    graph.replay()
+    assert torch.equal(acc.sum, want.sum) and torch.equal(acc.comp, want.comp)
